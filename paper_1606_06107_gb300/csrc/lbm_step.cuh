@@ -809,53 +809,169 @@ __global__ void LBM_STEP_BOUNDS k_step(const Params<Lattice<LAT>::Q, ST> p)
 }
 
 // ---------------------------------------------------------------------------
-// Initial state at equilibrium (pull pre-image in STREAM mode).
+// Initial state at equilibrium (pull pre-image in STREAM mode): population i
+// of node y is g_i^eq of the fields at bc(y + e_i).
+//
+// One thread evaluates its own node's equilibrium and writes population i to
+// every y with bc(y + e_i) = its node, so the nine polynomial coefficients
+// are formed once per node; the loads are the node's own fields and the
+// stores are shifted by at most three elements along the row.  (Evaluating at
+// the destination instead forms the coefficients once per population: on the
+// 2048^2 D2Q49 float state 910 us, on a 256^3 D3Q343 half state 33.5 ms.)
+// Bound by the stores' bandwidth in float (229 us, 940 MB at 2048^2: 0.60 of
+// the copy bandwidth) and by issue in half (150 us; D3Q343 4.39 ms).
+// A periodic axis is a bijection (one y per population); on a copy axis the
+// edge nodes also own the y whose y + e_i the clamp brings back to them (the
+// loop over ranges at the end) and nodes within three of an edge may own none.
+
+// Destinations lo..hi (none if lo > hi) of a node at x with velocity e on an
+// axis of n nodes: all y with bc(y + e) = x.
+struct PreImage {
+    int lo, hi;
+};
+__host__ __device__ __forceinline__ PreImage preimage(int x, int e, int n, int bc)
+{
+    PreImage r;
+    if (bc == 0) {
+        const int y = (((x - e) % n) + n) % n;
+        r.lo = r.hi = y;
+        return r;
+    }
+    r.lo = r.hi = x - e;
+    if (e >= 0 && x == n - 1) r.hi = n - 1;  // y + e past the end
+    if (e <= 0 && x == 0) r.lo = 0;          // y + e before the start
+    r.lo = r.lo < 0 ? 0 : r.lo;
+    r.hi = r.hi > n - 1 ? n - 1 : r.hi;
+    return r;
+}
 
 template <int LAT, bool ROT, int MODE, typename ST>
 __device__ __forceinline__ void init_node(const Params<Lattice<LAT>::Q, ST> &p, int x, int y, int z)
 {
     using L = Lattice<LAT>;
-    const int self = (z * p.Y + y) * p.pitch + x;
-    const float *rho_in = p.in0, *u_in = p.in1, *T_in = p.in2;
+    constexpr int Q = L::Q, D = L::D;
     constexpr bool is_node = NodeRef<ST>::value;
+    const int self = (z * p.Y + y) * p.pitch + x;
+    const int64_t node = ((int64_t)z * p.Y + y) * p.X + x;
+    const float rho = p.in0[node], T = p.in2[node];
+    const float ux = p.in1[node];
+    const float uy = (D >= 2) ? p.in1[p.N + node] : 0.f;
+    const float uz = (D >= 3) ? p.in1[2 * p.N + node] : 0.f;
+    const EqCoef k = eq_coef<D>(T, ux * ux + uy * uy + uz * uz, rho);
+    // the record of node `at` (per-node reference storage), from its own fields
+    auto record = [&](int64_t at) {
+        const float r0 = p.in0[at];
+        return make_float4(r0 - 1.0f, 0.5f * (r0 * (p.in2[at] - 1.0f)), r0 * (p.r * p.in1[at]),
+                           (D >= 2) ? r0 * (p.r * p.in1[p.N + at]) : 0.f);
+    };
+    // population i at the destination (dx, dy, dz)
+    auto put = [&](int i, int dx, int dy, int dz, float v) {
+        const int off = (dz * p.Y + dy) * p.pitch + dx;
+        if constexpr (is_node) st_ref(p, i, off, v, record(((int64_t)dz * p.Y + dy) * p.X + dx));
+        else st(p, i, off, v);
+    };
+    // (the same branch for the whole launch: a copy axis anywhere)
+    const bool open = MODE == 0 && (p.bc0 != 0 || (D >= 2 && p.bc1 != 0) || (D >= 3 && p.bc2 != 0));
+    // the one destination of each population (-1: outside a copy axis)
+    int ox[7], oy[7];  // destination of e = k - 3 along x and y
+    auto dest = [](int x, int e, int n, int bc) {
+        if (MODE != 0) return x;
+        if (bc == 0) return bc_wrap(x - e, n, 0);
+        return (x - e < 0 || x - e >= n) ? -1 : x - e;
+    };
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+        ox[j] = dest(x, j - 3, p.X, p.bc0);
+        oy[j] = (D >= 2) ? dest(y, j - 3, p.Y, p.bc1) : 0;
+    }
+    auto body = [&](auto checked) {
+        constexpr bool CHECK = decltype(checked)::value;
+        if constexpr (D < 3) {
+            // pairs of opposite velocities share the even and odd parts
+            static_for<0, (Q + 1) / 2>([&](auto ic) {
+                constexpr int I = decltype(ic)::value, J = Q - 1 - I;
+                constexpr int ex = L::ex(I), ey = L::ey(I);
+                const float c = p.r * ((float)ex * ux + (float)ey * uy + 0.f * uz);
+                float Pp, Pm;
+                eq_pair(k, c, p.r2 * (float)(ex * ex + ey * ey), Pp, Pm);
+                if (!CHECK || (ox[ex + 3] | oy[ey + 3]) >= 0) put(I, ox[ex + 3], oy[ey + 3], 0, p.w[I] * Pp);
+                if (I != J && (!CHECK || (ox[3 - ex] | oy[3 - ey]) >= 0))
+                    put(J, ox[3 - ex], oy[3 - ey], 0, p.w[J] * Pm);
+            });
+        } else {
+            // planes of e_z in a run-time loop (343 unrolled populations
+            // outgrow the instruction cache)
+#pragma unroll 1
+            for (int c7 = 0; c7 < 7; ++c7) {
+                const int ez = c7 - 3;
+                const int dz = dest(z, ez, p.Z, p.bc2);
+#pragma unroll
+                for (int j = 0; j < 49; ++j) {
+                    const int ex = j % 7 - 3, ey = j / 7 - 3;
+                    const float c = p.r * ((float)ex * ux + (float)ey * uy + (float)ez * uz);
+                    const float s = p.r2 * (float)(ex * ex + ey * ey + ez * ez);
+                    if (!CHECK || (ox[ex + 3] | oy[ey + 3] | dz) >= 0)
+                        put(c7 * 49 + j, ox[ex + 3], oy[ey + 3], dz, p.w[c7 * 49 + j] * eq_single(k, c, s));
+                }
+            }
+        }
+    };
+    if (!open) {
+        body(std::false_type{});
+    } else {
+        body(std::true_type{});
+        // the further destinations of a node on a copy axis's end, for the
+        // velocities that point out of it
+        const bool xl = p.bc0 != 0 && x == 0, xh = p.bc0 != 0 && x == p.X - 1;
+        const bool yl = D >= 2 && p.bc1 != 0 && y == 0, yh = D >= 2 && p.bc1 != 0 && y == p.Y - 1;
+        const bool zl = D >= 3 && p.bc2 != 0 && z == 0, zh = D >= 3 && p.bc2 != 0 && z == p.Z - 1;
+        auto spread = [&](int i, int ex, int ey, int ez) {
+            if (!((xl && ex < 0) || (xh && ex > 0) || (yl && ey < 0) || (yh && ey > 0) || (zl && ez < 0) ||
+                  (zh && ez > 0)))
+                return;
+            const PreImage rx = preimage(x, ex, p.X, p.bc0);
+            const PreImage ry = (D >= 2) ? preimage(y, ey, p.Y, p.bc1) : PreImage{0, 0};
+            const PreImage rz = (D >= 3) ? preimage(z, ez, p.Z, p.bc2) : PreImage{0, 0};
+            const float c = p.r * ((float)ex * ux + (float)ey * uy + (float)ez * uz);
+            const float v = p.w[i] * eq_single(k, c, p.r2 * (float)(ex * ex + ey * ey + ez * ez));
+#pragma unroll 1
+            for (int dz = rz.lo; dz <= rz.hi; ++dz)
+#pragma unroll 1
+                for (int dy = ry.lo; dy <= ry.hi; ++dy)
+#pragma unroll 1
+                    for (int dx = rx.lo; dx <= rx.hi; ++dx) put(i, dx, dy, dz, v);
+        };
+        if (xl || xh || yl || yh || zl || zh) {
+            // (7 populations unrolled: the ensemble's parameters are a
+            // register copy, which a run-time index would send to local
+            // memory; 37 and 49 unrolled cost more in cold instructions than
+            // the loops do, and so does a velocity table in cold memory)
+            if constexpr (Q == 7) {
+                static_for<0, Q>([&](auto ic) { spread(decltype(ic)::value, L::ex(decltype(ic)::value), 0, 0); });
+            } else {
+                int i = 0;
+#pragma unroll 1
+                for (int ez = (D >= 3) ? -3 : 0; ez <= ((D >= 3) ? 3 : 0); ++ez)
+#pragma unroll 1
+                    for (int ey = -3; ey <= 3; ++ey)
+#pragma unroll 1
+                        for (int ex = -3; ex <= 3; ++ex)
+                            if (Q != 37 || d2q37_member(ex, ey)) spread(i++, ex, ey, ez);
+            }
+        }
+    }
     float4 rc = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (is_node) {  // the node's reference: its own initial fields
-        const int64_t node = ((int64_t)z * p.Y + y) * p.X + x;
-        const float r0 = rho_in[node];
-        rc = make_float4(r0 - 1.0f, 0.5f * (r0 * (T_in[node] - 1.0f)), r0 * (p.r * u_in[node]),
-                         (L::D >= 2) ? r0 * (p.r * u_in[p.N + node]) : 0.f);
+        rc = record(node);
         p.ref_dst[self] = rc;
     }
-#pragma unroll 1
-    for (int i = 0; i < L::Q; ++i) {
-        const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
-        int sx = x, sy = y, sz = z;
-        if (MODE == 0) {
-            sx = bc_wrap(x + ex, p.X, p.bc0);
-            if (L::D >= 2) sy = bc_wrap(y + ey, p.Y, p.bc1);
-            if (L::D >= 3) sz = bc_wrap(z + ez, p.Z, p.bc2);
-        }
-        const int64_t src = ((int64_t)sz * p.Y + sy) * p.X + sx;
-        const float rho = rho_in[src];
-        const float ux = u_in[src];
-        const float uy = (L::D >= 2) ? u_in[p.N + src] : 0.f;
-        const float uz = (L::D >= 3) ? u_in[2 * p.N + src] : 0.f;
-        const float T = T_in[src];
-        const EqCoef k = eq_coef<L::D>(T, ux * ux + uy * uy + uz * uz, rho);
-        const float c = p.r * ((float)ex * ux + (float)ey * uy + (float)ez * uz);
-        const float s = p.r2 * (float)(ex * ex + ey * ey + ez * ez);
-        if constexpr (is_node) st_ref(p, i, self, p.w[i] * eq_single(k, c, s), rc);
-        else st(p, i, self, p.w[i] * eq_single(k, c, s));
-    }
     if (ROT) {
-        const int64_t node = ((int64_t)z * p.Y + y) * p.X + x;
         float heq[7];
-        const float Tn = T_in[node];
-        heq_node(p, Tn, Tn * p.inv_r2, heq);
+        heq_node(p, T, T * p.inv_r2, heq);
 #pragma unroll
         for (int j = 0; j < 7; ++j) {
-            if constexpr (is_node) st_ref(p, L::Q + j, self, heq[j], rc);
-            else st(p, L::Q + j, self, heq[j]);
+            if constexpr (is_node) st_ref(p, Q + j, self, heq[j], rc);
+            else st(p, Q + j, self, heq[j]);
         }
     }
 }
@@ -1009,6 +1125,7 @@ __global__ void __launch_bounds__(kBlockX) k_set_state(const Params<Lattice<LAT>
 
 // The D3Q343 step (lbm_d3q343.cu): STREAM transport only.
 template <bool ROT, typename ST> cudaError_t launch_step_q343(const Args &a, cudaStream_t s);
+template <bool ROT, typename ST> cudaError_t launch_moments_q343(const Args &a, cudaStream_t s);
 
 template <int LAT, bool ROT, int MODE, typename ST>
 cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
@@ -1028,7 +1145,10 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
         }
         break;
     case Op::Init: k_init<LAT, ROT, MODE><<<grid, block, 0, s>>>(p); break;
-    case Op::Moments: k_moments<LAT, ROT, MODE><<<grid, block, 0, s>>>(p); break;
+    case Op::Moments:
+        if constexpr (LAT == 4) return launch_moments_q343<ROT, ST>(a, s);
+        else k_moments<LAT, ROT, MODE><<<grid, block, 0, s>>>(p);
+        break;
     case Op::Conserve: k_conserve<LAT, ROT, MODE><<<a.red_blocks, kRedThreads, 0, s>>>(p); break;
     case Op::GetState: k_get_state<LAT, ROT><<<grid, block, 0, s>>>(p); break;
     case Op::SetState: k_set_state<LAT, ROT><<<grid, block, 0, s>>>(p); break;
