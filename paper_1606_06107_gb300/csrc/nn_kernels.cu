@@ -1126,115 +1126,304 @@ __global__ void k_lift(const float *feat, const float *Wl, const float *bl, __nv
     }
 }
 
-// out[p][o] = sum_c x[p][c] Wp[o][c] + bp[o]: one thread per position reads
-// its row of C bf16 values as 16-byte vectors; the FO x C weights sit in
-// shared memory and are read as warp-wide broadcasts.
-template <int FO>
-__global__ void k_head(const __nv_bfloat16 *x, const float *Wp, const float *bp, float *out,
-                       int64_t P, int C)
+// Two floats in a register pair and one fused multiply-add on both: the same
+// rounding as two scalar ones in half the issue slots.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
 {
-    extern __shared__ float wsh[];  // [FO][C]
-    for (int i = threadIdx.x; i < FO * C; i += blockDim.x) wsh[i] = Wp[i];
-    __syncthreads();
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    float acc[FO];
-#pragma unroll
-    for (int o = 0; o < FO; ++o) acc[o] = __ldg(bp + o);
-    const uint4 *row = reinterpret_cast<const uint4 *>(x + p * C);
-    for (int c8 = 0; c8 < C / 8; ++c8) {
-        float xv[8];
-        unpack8(__ldg(row + c8), xv);
-#pragma unroll
-        for (int o = 0; o < FO; ++o) {
-            const float4 w0 = *reinterpret_cast<const float4 *>(wsh + o * C + 8 * c8);
-            const float4 w1 = *reinterpret_cast<const float4 *>(wsh + o * C + 8 * c8 + 4);
-            acc[o] = fmaf(xv[0], w0.x, acc[o]);
-            acc[o] = fmaf(xv[1], w0.y, acc[o]);
-            acc[o] = fmaf(xv[2], w0.z, acc[o]);
-            acc[o] = fmaf(xv[3], w0.w, acc[o]);
-            acc[o] = fmaf(xv[4], w1.x, acc[o]);
-            acc[o] = fmaf(xv[5], w1.y, acc[o]);
-            acc[o] = fmaf(xv[6], w1.z, acc[o]);
-            acc[o] = fmaf(xv[7], w1.w, acc[o]);
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr(dst)), "l"(src) : "memory");
+}
+
+// out[p][o] = sum_c x[p][c] Wp[o][c] + bp[o]: a block of 128 threads takes
+// 128 NP positions (NP a thread, 128 apart).  Their rows come through shared
+// memory, 32 channels at a time, two chunks in flight (cp.async): a thread
+// that reads its own row from global memory takes 16 bytes of a line that is
+// evicted before its next read.  The weights sit in shared memory channel by
+// channel ([C][FO], FO rounded up to even) so that one broadcast read gives
+// the weights of two or four outputs, which one packed multiply-add each then
+// serves.  Every output is still summed over c in ascending order.  Bound by
+// the multiply-adds (40 us at 2^20 positions, 12 outputs) next to the 268 MB
+// of x: 127 us (160 with each thread on its own row in global memory).
+constexpr int kHeadChunk = 32;                    // channels per staged chunk
+constexpr int kHeadPitch = kHeadChunk * 2 + 16;   // bytes per staged row: conflict-free 16-byte reads
+template <int FO, int NP>
+__global__ void __launch_bounds__(128)
+    k_head(const __nv_bfloat16 *x, const float *Wp, const float *bp, float *out, int64_t P, int C)
+{
+    constexpr int FP = (FO + 1) / 2 * 2, kRows = 128 * NP;
+    extern __shared__ float4 wsh4[];  // [2][kRows][kHeadPitch] staged rows, [C][FP] weights
+    uint8_t *rows = reinterpret_cast<uint8_t *>(wsh4);
+    float *wsh = reinterpret_cast<float *>(rows + 2 * kRows * kHeadPitch);
+    const int64_t first = (int64_t)blockIdx.x * kRows;
+    const int chunks = (C + kHeadChunk - 1) / kHeadChunk;
+    auto fetch = [&](int k) {
+        uint8_t *dst = rows + (k & 1) * kRows * kHeadPitch;
+        const int vecs = min((int)kHeadChunk, C - k * (int)kHeadChunk) / 8;  // 16-byte vectors of a row (C % 8 == 0)
+        for (int e = threadIdx.x; e < kRows * 4; e += 128) {
+            const int r = e >> 2, v = e & 3;
+            if (v < vecs && first + r < P)
+                cp_async16(dst + r * kHeadPitch + 16 * v, x + (first + r) * C + k * kHeadChunk + 8 * v);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(0);
+    for (int i = threadIdx.x; i < FP * C; i += blockDim.x) {
+        const int o = i / C, c = i % C;
+        wsh[c * FP + o] = o < FO ? Wp[i] : 0.f;
+    }
+    uint64_t acc[NP][FP / 2];
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+#pragma unroll
+        for (int o = 0; o < FP; o += 2) acc[q][o / 2] = pack2(__ldg(bp + o), o + 1 < FO ? __ldg(bp + o + 1) : 0.f);
+    for (int k = 0; k < chunks; ++k) {
+        if (k + 1 < chunks) {
+            fetch(k + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const uint8_t *src = rows + (k & 1) * kRows * kHeadPitch + threadIdx.x * kHeadPitch;
+        const int vecs = min((int)kHeadChunk, C - k * (int)kHeadChunk) / 8;
+#pragma unroll 1
+        for (int v = 0; v < vecs; ++v) {
+            float xv[NP][8];
+#pragma unroll
+            for (int q = 0; q < NP; ++q)
+                unpack8(*reinterpret_cast<const uint4 *>(src + q * 128 * kHeadPitch + 16 * v), xv[q]);
+            const float *wc = wsh + (k * kHeadChunk + 8 * v) * FP;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float *w = wc + j * FP;
+                uint64_t wv[FP / 2];
+                if constexpr (FP % 4 == 0) {
+#pragma unroll
+                    for (int o = 0; o < FP / 4; ++o) {
+                        const ulonglong2 t = reinterpret_cast<const ulonglong2 *>(w)[o];
+                        wv[2 * o] = t.x, wv[2 * o + 1] = t.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int o = 0; o < FP / 2; ++o) wv[o] = reinterpret_cast<const unsigned long long *>(w)[o];
+                }
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    const uint64_t xx = pack2(xv[q][j], xv[q][j]);
+#pragma unroll
+                    for (int o = 0; o < FP / 2; ++o) acc[q][o] = fma2(xx, wv[o], acc[q][o]);
+                }
+            }
+        }
+        __syncthreads();  // this chunk's buffer is refilled two chunks on
     }
 #pragma unroll
-    for (int o = 0; o < FO; ++o) out[p * FO + o] = acc[o];
+    for (int q = 0; q < NP; ++q) {
+        const int64_t p = first + q * 128 + threadIdx.x;
+        if (p >= P) continue;
+#pragma unroll
+        for (int o = 0; o < FP; o += 2) {
+            float a, b;
+            unpack2(acc[q][o / 2], a, b);
+            out[p * FO + o] = a;
+            if (o + 1 < FO) out[p * FO + o + 1] = b;
+        }
+    }
 }
 
 // Head backward: gx = gout Wp; gz = bf16(gx gelu'(z)); gWp += gout^T x; gbp += sum gout.
-// One warp per position, lane holding channels lane + 32 j (NJ = C / 32),
-// FO outputs: both compile-time so that the partial sums stay in registers
-// (the head weights are read through L1).
-template <int NJ, int FO>
-__global__ void k_head_bwd(const float *gout, const __nv_bfloat16 *x, const float *Wp,
-                           const __nv_bfloat16 *z, float *gx, __nv_bfloat16 *gz, float *gWp,
-                           float *gbp, int64_t P)
+// One warp per position, FO outputs, NJ = C / 32 channels a lane, both
+// compile-time so that the partial sums stay in registers.  VEC: a lane holds
+// four consecutive channels (16-byte aligned tensors), so a row is read and
+// written in whole vectors; else channels lane + 32 j.  A block first adds up
+// its warps' partial sums in shared memory and then makes one coalesced
+// reduction into gWp: with one reduction per warp the same-address traffic
+// (7.5 M reductions into 1536 addresses) was the kernel: 36 us at 2^15
+// positions, C = 128, FO = 12 (103 before).
+template <int NJ, int FO, bool VEC>
+__global__ void __launch_bounds__(256) k_head_bwd(const float *gout, const __nv_bfloat16 *x, const float *Wp,
+                                                  const __nv_bfloat16 *z, float *gx, __nv_bfloat16 *gz,
+                                                  float *gWp, float *gbp, int64_t P)
 {
     constexpr int C = 32 * NJ;
-    const int lane = threadIdx.x & 31;
+    constexpr bool WREG = FO * NJ <= 48;  // the weights fit in registers beside the sums
+    __shared__ float red[FO * C + FO];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    float accW[FO][NJ], accB[FO];
+    auto chan = [&](int j) { return VEC ? 4 * lane + (j & 3) + 128 * (j >> 2) : lane + 32 * j; };
+    float accW[FO][NJ], accB[FO], w[WREG ? FO : 1][NJ];
 #pragma unroll
     for (int o = 0; o < FO; ++o) {
         accB[o] = 0.f;
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) accW[o][j] = 0.f;
+        for (int j = 0; j < NJ; ++j) {
+            accW[o][j] = 0.f;
+            if constexpr (WREG) w[o][j] = __ldg(Wp + o * C + chan(j));
+        }
     }
-    for (int64_t p = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); p < P; p += warps) {
+    // the next position's values are in flight while one is worked on
+    struct Row {
         float go[FO];
+        uint2 xq[VEC ? NJ / 4 : 1], zq[VEC ? NJ / 4 : 1];
+        __nv_bfloat16 xs[VEC ? 1 : NJ], zs[VEC ? 1 : NJ];
+    } next;
+    auto fetch = [&](int64_t p) {
+#pragma unroll
+        for (int o = 0; o < FO; ++o) next.go[o] = __ldg(gout + p * FO + o);
+        if constexpr (VEC) {
+#pragma unroll
+            for (int v = 0; v < NJ / 4; ++v) {
+                const int64_t c = p * C + 4 * lane + 128 * v;
+                next.xq[v] = __ldg(reinterpret_cast<const uint2 *>(x + c));
+                next.zq[v] = __ldg(reinterpret_cast<const uint2 *>(z + c));
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                next.xs[j] = x[p * C + chan(j)];
+                next.zs[j] = z[p * C + chan(j)];
+            }
+        }
+    };
+    int64_t p = blockIdx.x * (int64_t)(blockDim.x >> 5) + warp;
+    if (p < P) fetch(p);
+    for (; p < P; p += warps) {
+        float go[FO], xv[NJ], zv[NJ], g[NJ];
 #pragma unroll
         for (int o = 0; o < FO; ++o) {
-            go[o] = __ldg(gout + p * FO + o);
+            go[o] = next.go[o];
             accB[o] += go[o];
         }
+        if constexpr (VEC) {
+#pragma unroll
+            for (int v = 0; v < NJ / 4; ++v) {
+                const float2 x0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&next.xq[v].x));
+                const float2 x1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&next.xq[v].y));
+                const float2 z0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&next.zq[v].x));
+                const float2 z1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&next.zq[v].y));
+                xv[4 * v] = x0.x, xv[4 * v + 1] = x0.y, xv[4 * v + 2] = x1.x, xv[4 * v + 3] = x1.y;
+                zv[4 * v] = z0.x, zv[4 * v + 1] = z0.y, zv[4 * v + 2] = z1.x, zv[4 * v + 3] = z1.y;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                xv[j] = __bfloat162float(next.xs[j]);
+                zv[j] = __bfloat162float(next.zs[j]);
+            }
+        }
+        if (p + warps < P) fetch(p + warps);
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
-            const int64_t c = p * C + lane + 32 * j;
-            const float xv = __bfloat162float(x[c]);
-            float g = 0.f;
+            g[j] = 0.f;
 #pragma unroll
             for (int o = 0; o < FO; ++o) {
-                g = fmaf(go[o], __ldg(Wp + o * C + lane + 32 * j), g);
-                accW[o][j] = fmaf(go[o], xv, accW[o][j]);
+                g[j] = fmaf(go[o], WREG ? w[WREG ? o : 0][j] : __ldg(Wp + o * C + chan(j)), g[j]);
+                accW[o][j] = fmaf(go[o], xv[j], accW[o][j]);
             }
-            gx[c] = g;
-            gz[c] = __float2bfloat16_rn(g * gelu_grad(__bfloat162float(z[c])));
+        }
+        if constexpr (VEC) {
+#pragma unroll
+            for (int v = 0; v < NJ / 4; ++v) {
+                const int64_t c = p * C + 4 * lane + 128 * v;
+                *reinterpret_cast<float4 *>(gx + c) = make_float4(g[4 * v], g[4 * v + 1], g[4 * v + 2], g[4 * v + 3]);
+                uint2 q;
+                *reinterpret_cast<__nv_bfloat162 *>(&q.x) = __floats2bfloat162_rn(
+                    g[4 * v] * gelu_grad(zv[4 * v]), g[4 * v + 1] * gelu_grad(zv[4 * v + 1]));
+                *reinterpret_cast<__nv_bfloat162 *>(&q.y) = __floats2bfloat162_rn(
+                    g[4 * v + 2] * gelu_grad(zv[4 * v + 2]), g[4 * v + 3] * gelu_grad(zv[4 * v + 3]));
+                *reinterpret_cast<uint2 *>(gz + c) = q;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                gx[p * C + chan(j)] = g[j];
+                gz[p * C + chan(j)] = __float2bfloat16_rn(g[j] * gelu_grad(zv[j]));
+            }
         }
     }
+    // the block's sums: its warps in turn
+    for (int wi = 0; wi < (int)(blockDim.x >> 5); ++wi) {
+        if (warp == wi) {
 #pragma unroll
-    for (int o = 0; o < FO; ++o) {
+            for (int o = 0; o < FO; ++o) {
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) atomicAdd(&gWp[o * C + lane + 32 * j], accW[o][j]);
-        if (lane == 0) atomicAdd(&gbp[o], accB[o]);
+                for (int j = 0; j < NJ; ++j) {
+                    float *r = red + o * C + chan(j);
+                    *r = wi ? *r + accW[o][j] : accW[o][j];
+                }
+                if (lane == 0) red[FO * C + o] = wi ? red[FO * C + o] + accB[o] : accB[o];
+            }
+        }
+        __syncthreads();
     }
+    for (int i = threadIdx.x; i < FO * C; i += blockDim.x) atomicAdd(gWp + i, red[i]);
+    if (threadIdx.x < FO) atomicAdd(gbp + threadIdx.x, red[FO * C + threadIdx.x]);
 }
 
 // Lift backward: gWl[c][j] += sum_p gx0[p][c] feat[p][j]; gbl[c] += sum_p gx0[p][c].
-// Threads over channels, blocks over position ranges, F features compile-time.
+// R = blockDim / C groups of C threads take the block's positions in turn
+// (thread = channel, the features broadcast from shared memory), their sums
+// meet in shared memory and leave as one coalesced reduction per block.
+// Bound by the read of gx0; with one strided reduction per thread and the
+// features read through L1 it was latency and same-address traffic: 27 us at
+// 2^15 positions, C = 128, F = 16 (82 before).
 template <int F>
-__global__ void k_lift_bwd(const float *gx0, const float *feat, float *gWl, float *gbl, int64_t P,
-                           int C, int64_t per_block)
+__global__ void __launch_bounds__(1024) k_lift_bwd(const float *gx0, const float *feat, float *gWl, float *gbl,
+                                                   int64_t P, int C, int per_block)
 {
-    const int c = threadIdx.x;  // blockDim.x == C
-    float acc[F];
+    extern __shared__ float4 lsh4[];
+    float *sh = reinterpret_cast<float *>(lsh4);  // [per_block][F], then [C][F] and [C]
+    const int c = threadIdx.x % C, r = threadIdx.x / C, R = blockDim.x / C;
+    const int64_t p0 = (int64_t)blockIdx.x * per_block;
+    const int n = (int)std::min<int64_t>(per_block, P - p0);
+    for (int e = threadIdx.x; e < n * F; e += blockDim.x) sh[e] = __ldg(feat + p0 * F + e);
+    __syncthreads();
+    float acc[F], accb = 0.f;
 #pragma unroll
     for (int j = 0; j < F; ++j) acc[j] = 0.f;
-    float accb = 0.f;
-    const int64_t p0 = blockIdx.x * per_block, p1 = std::min(P, p0 + per_block);
-    for (int64_t p = p0; p < p1; ++p) {
-        const float g = gx0[p * C + c];
+#pragma unroll 8
+    for (int q = r; q < n; q += R) {
+        const float g = __ldg(gx0 + (p0 + q) * C + c);
         accb += g;
 #pragma unroll
-        for (int j = 0; j < F; ++j) acc[j] = fmaf(g, __ldg(feat + p * F + j), acc[j]);
+        for (int j = 0; j < F / 4; ++j) {
+            const float4 f = lsh4[q * (F / 4) + j];
+            acc[4 * j] = fmaf(g, f.x, acc[4 * j]);
+            acc[4 * j + 1] = fmaf(g, f.y, acc[4 * j + 1]);
+            acc[4 * j + 2] = fmaf(g, f.z, acc[4 * j + 2]);
+            acc[4 * j + 3] = fmaf(g, f.w, acc[4 * j + 3]);
+        }
     }
+    __syncthreads();  // the features have been read
+    for (int k = 0; k < R; ++k) {
+        if (r == k) {
 #pragma unroll
-    for (int j = 0; j < F; ++j) atomicAdd(&gWl[c * F + j], acc[j]);
-    atomicAdd(&gbl[c], accb);
+            for (int j = 0; j < F; ++j) sh[c * F + j] = k ? sh[c * F + j] + acc[j] : acc[j];
+            sh[C * F + c] = k ? sh[C * F + c] + accb : accb;
+        }
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < C * F; e += blockDim.x) atomicAdd(gWl + e, sh[e]);
+    for (int e = threadIdx.x; e < C; e += blockDim.x) atomicAdd(gbl + e, sh[C * F + e]);
 }
 
-// gb[c] += sum_p gz[p][c] (bf16 input), threads over channels
+// gb[c] += sum_p gz[p][c] (bf16 input), threads over channels: any C.
 __global__ void k_colsum(const __nv_bfloat16 *gz, float *gb, int64_t P, int C, int64_t per_block)
 {
     const int64_t p0 = blockIdx.x * per_block, p1 = std::min(P, p0 + per_block);
@@ -1242,6 +1431,38 @@ __global__ void k_colsum(const __nv_bfloat16 *gz, float *gb, int64_t P, int C, i
         float s = 0.f;
         for (int64_t p = p0; p < p1; ++p) s += __bfloat162float(gz[p * C + c]);
         atomicAdd(&gb[c], s);
+    }
+}
+
+// The same for C a multiple of 128 and an aligned tensor: 16 threads read a
+// row's 128 channels as 16-byte vectors, 16 rows at a time, and the block's
+// sums meet in shared memory.  Bound by the read; the form above reads two
+// bytes a thread in one serial chain: 6.5 us at 2^15 x 128 (10.9 before).
+__global__ void __launch_bounds__(256) k_colsum8(const __nv_bfloat16 *gz, float *gb, int64_t P, int C,
+                                                 int64_t per_block)
+{
+    __shared__ float red[16][kTile + 4];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int64_t p0 = blockIdx.x * per_block, p1 = std::min(P, p0 + per_block);
+    const __nv_bfloat16 *base = gz + blockIdx.y * kTile + 8 * tx;
+    float s[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] = 0.f;
+#pragma unroll 8
+    for (int64_t p = p0 + ty; p < p1; p += 16) {
+        float v[8];
+        unpack8(__ldg(reinterpret_cast<const uint4 *>(base + p * C)), v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] += v[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) red[ty][8 * tx + j] = s[j];
+    __syncthreads();
+    if (threadIdx.x < kTile) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) t += red[k][threadIdx.x];
+        atomicAdd(&gb[blockIdx.y * kTile + threadIdx.x], t);
     }
 }
 
@@ -1333,9 +1554,10 @@ __global__ void k_sample_pairs(const int *good, int ngood, int windows, int tube
 __global__ void k_mse(const float *out, const float *target, float *gout, double *loss, int64_t n)
 {
     double acc = 0.0;
+#pragma unroll 4
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float d = out[i] - target[i];
+        const float d = __ldg(out + i) - __ldg(target + i);
         acc += (double)d * d;
         if (gout) gout[i] = 2.0f * d / (float)n;
     }
@@ -1594,6 +1816,27 @@ int set_smem_attrs()
     return LBM_OK;
 }
 
+// once per device: the head's dynamic shared memory (two staged chunks of up
+// to 256 rows and 48 KB of weights)
+int set_head_attrs()
+{
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LBM_ECUDA;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done[dev]) return LBM_OK;
+    const void *fn[] = {(const void *)k_head<3, 1>,  (const void *)k_head<3, 2>,  (const void *)k_head<6, 1>,
+                        (const void *)k_head<6, 2>,  (const void *)k_head<12, 1>, (const void *)k_head<12, 2>,
+                        (const void *)k_head<24, 1>, (const void *)k_head<24, 2>};
+    for (const void *f : fn)
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 48 * 1024 + 2 * 256 * kHeadPitch) != cudaSuccess)
+            return LBM_ECUDA;
+    done[dev] = true;
+    return LBM_OK;
+}
+
 int launched(cudaError_t e) { return e == cudaSuccess ? LBM_OK : LBM_ECUDA; }
 
 bool conv_shape_ok(int B, int L, int C, int k, int dil, int impl)
@@ -1781,14 +2024,26 @@ int lbm_nn_lift_backward(const float *gx0, const float *feat, float *gWl, float 
     if (!gx0 || !feat || !gWl || !gbl || P < 1 || C < 32 || C > 1024 || C % 32 ||
         (F != 4 && F != 8 && F != 16 && F != 32))
         return LBM_EINVAL;
-    const int64_t per_block = std::max<int64_t>(64, (P + 1215) / 1216);
-    const int blocks = (int)((P + per_block - 1) / per_block);
+    // 128 positions a block keep two blocks on every SM from 2^15 positions
+    // on; more of them for larger P, so that the reductions stay few
+    const int64_t want = std::max<int64_t>(128, (P + 8 * 152 - 1) / (8 * 152));
+    const int per_block = (int)std::min<int64_t>(want, 16384 / (F * 4) * 2);  // features: at most 32 KB
+    const int64_t nblocks = (P + per_block - 1) / per_block;
+    if (nblocks > 0x7fffffff) return LBM_EINVAL;
+    const int blocks = (int)nblocks, threads = C * std::max(1, 512 / C);
+    const size_t sh = sizeof(float) * std::max((size_t)per_block * F, (size_t)C * (F + 1));
     cudaStream_t s = (cudaStream_t)stream;
+    // [C][F + 1] sums of 1024 channels and 32 features exceed 48 KB
+    const void *fn = F == 4 ? (const void *)k_lift_bwd<4> : F == 8 ? (const void *)k_lift_bwd<8>
+                   : F == 16 ? (const void *)k_lift_bwd<16> : (const void *)k_lift_bwd<32>;
+    if (sh > 48 * 1024 &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh) != cudaSuccess)
+        return LBM_ECUDA;
     switch (F) {
-    case 4: k_lift_bwd<4><<<blocks, C, 0, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
-    case 8: k_lift_bwd<8><<<blocks, C, 0, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
-    case 16: k_lift_bwd<16><<<blocks, C, 0, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
-    default: k_lift_bwd<32><<<blocks, C, 0, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
+    case 4: k_lift_bwd<4><<<blocks, threads, sh, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
+    case 8: k_lift_bwd<8><<<blocks, threads, sh, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
+    case 16: k_lift_bwd<16><<<blocks, threads, sh, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
+    default: k_lift_bwd<32><<<blocks, threads, sh, s>>>(gx0, feat, gWl, gbl, P, C, per_block); break;
     }
     return launched(cudaGetLastError());
 }
@@ -1799,15 +2054,28 @@ int lbm_nn_head(const void *x, const float *Wp, const float *bp, float *out, int
     if (!x || !Wp || !bp || !out || P < 1 || C < 8 || C > 1024 || C % 8 || !aligned16(x) ||
         !aligned16(Wp) || (Fo != 3 && Fo != 6 && Fo != 12 && Fo != 24))
         return LBM_EINVAL;
-    const int64_t nblocks = (P + 127) / 128;
+    // two positions a thread halve the weight reads; one while two would
+    // leave SMs without a second block
+    const bool two = P >= 2 * 256 * 152;
+    const int64_t nblocks = two ? (P + 255) / 256 : (P + 127) / 128;
     if (nblocks > 0x7fffffff) return LBM_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     auto xb = (const __nv_bfloat16 *)x;
-    const size_t sh = sizeof(float) * Fo * C;
-    if (Fo == 3) k_head<3><<<(int)nblocks, 128, sh, s>>>(xb, Wp, bp, out, P, C);
-    else if (Fo == 6) k_head<6><<<(int)nblocks, 128, sh, s>>>(xb, Wp, bp, out, P, C);
-    else if (Fo == 12) k_head<12><<<(int)nblocks, 128, sh, s>>>(xb, Wp, bp, out, P, C);
-    else k_head<24><<<(int)nblocks, 128, sh, s>>>(xb, Wp, bp, out, P, C);
+    const size_t wbytes = sizeof(float) * ((Fo + 1) / 2 * 2) * C, row2 = 2 * 128 * kHeadPitch;
+    if (wbytes > 48 * 1024) return LBM_ECUDA;  // as before: 48 KB of weights at most
+    const size_t sh = wbytes + (two ? 2 : 1) * row2;
+    int rc = set_head_attrs();
+    if (rc != LBM_OK) return rc;
+#define LBM_HEAD(FO)                                                                     \
+    do {                                                                                 \
+        if (two) k_head<FO, 2><<<(int)nblocks, 128, sh, s>>>(xb, Wp, bp, out, P, C);     \
+        else k_head<FO, 1><<<(int)nblocks, 128, sh, s>>>(xb, Wp, bp, out, P, C);         \
+    } while (0)
+    if (Fo == 3) LBM_HEAD(3);
+    else if (Fo == 6) LBM_HEAD(6);
+    else if (Fo == 12) LBM_HEAD(12);
+    else LBM_HEAD(24);
+#undef LBM_HEAD
     return launched(cudaGetLastError());
 }
 
@@ -1817,13 +2085,18 @@ int lbm_nn_head_backward(const float *gout, const void *x, const float *Wp, cons
     if (!gout || !x || !Wp || !z || !gx || !gz || !gWp || !gbp || P < 1 ||
         (C != 128 && C != 256) || (Fo != 3 && Fo != 6 && Fo != 12 && Fo != 24))
         return LBM_EINVAL;
-    const int grid = (int)std::min<int64_t>(grid_for(P * 32), 152 * 4);
+    // two blocks an SM: enough warps to hide the loads, few reductions
+    const int grid = (int)std::min<int64_t>((P + 7) / 8, 152 * 2);
+    const bool vec = aligned16(x) && aligned16(z) && aligned16(gx) && aligned16(gz);
     cudaStream_t s = (cudaStream_t)stream;
     auto xb = (const __nv_bfloat16 *)x;
     auto zb = (const __nv_bfloat16 *)z;
     auto gzb = (__nv_bfloat16 *)gz;
-#define LBM_HEAD_BWD(NJ, FO) \
-    k_head_bwd<NJ, FO><<<grid, 256, 0, s>>>(gout, xb, Wp, zb, gx, gzb, gWp, gbp, P)
+#define LBM_HEAD_BWD(NJ, FO)                                                                          \
+    do {                                                                                              \
+        if (vec) k_head_bwd<NJ, FO, true><<<grid, 256, 0, s>>>(gout, xb, Wp, zb, gx, gzb, gWp, gbp, P); \
+        else k_head_bwd<NJ, FO, false><<<grid, 256, 0, s>>>(gout, xb, Wp, zb, gx, gzb, gWp, gbp, P);    \
+    } while (0)
     if (C == 128) {
         if (Fo == 3) LBM_HEAD_BWD(4, 3);
         else if (Fo == 6) LBM_HEAD_BWD(4, 6);
@@ -1842,6 +2115,13 @@ int lbm_nn_head_backward(const float *gout, const void *x, const float *Wp, cons
 int lbm_nn_bias_grad(const void *gz, float *gb, int64_t P, int C, void *stream)
 {
     if (!gz || !gb || P < 1 || C < 1) return LBM_EINVAL;
+    if (C % kTile == 0 && C / kTile <= 65535 && aligned16(gz)) {
+        // about two blocks an SM, at least four rows a thread
+        const int64_t rows = std::max<int64_t>(64, (P * (C / kTile) + 303) / 304);
+        const dim3 grid((unsigned)((P + rows - 1) / rows), C / kTile);
+        k_colsum8<<<grid, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16 *)gz, gb, P, C, rows);
+        return launched(cudaGetLastError());
+    }
     const int64_t per_block = std::max<int64_t>(64, (P + 1215) / 1216);
     const int blocks = (int)((P + per_block - 1) / per_block);
     k_colsum<<<blocks, std::min(C, 256), 0, (cudaStream_t)stream>>>((const __nv_bfloat16 *)gz, gb, P,
@@ -1890,7 +2170,8 @@ int lbm_nn_mse(const float *out, const float *target, float *gout, double *loss,
                void *stream)
 {
     if (!out || !target || !loss || n < 1) return LBM_EINVAL;
-    k_mse<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(out, target, gout, loss, n);
+    // few blocks: each ends in one double-precision reduction into `loss`
+    k_mse<<<std::min(grid_for(n), 304), 256, 0, (cudaStream_t)stream>>>(out, target, gout, loss, n);
     return launched(cudaGetLastError());
 }
 
