@@ -498,6 +498,17 @@ int lbm_step(lbm_handle h, int64_t k)
     if (!h->has_state) return fail(h, LBM_ESTATE, "no state: call lbm_set_macro or lbm_set_state");
     DeviceGuard g(h->device);
     Args a = make_args(h);
+    if (h->lattice == LBM_D1Q7 && lbm::tube_steps_ok(a, k)) {
+        const int end = h->cur ^ (int)(k & 1);  // the buffer single steps would end in
+        a.src = h->buf[h->cur];
+        a.dst = h->buf[end];
+        ++h->launches;
+        const cudaError_t e = lbm::launch_tube_steps(a, k, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "tube kernel");
+        h->cur = end;
+        h->steps += k;
+        return LBM_OK;
+    }
     for (int64_t s = 0; s < k; ++s) {
         a.src = static_cast<const float *>(h->buf[h->cur]);
         a.dst = static_cast<float *>(h->buf[h->cur ^ 1]);

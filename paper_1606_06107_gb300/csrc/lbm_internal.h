@@ -49,4 +49,9 @@ cudaError_t launch_d2q37(Op op, const Args &a, cudaStream_t s);
 cudaError_t launch_d2q49(Op op, const Args &a, cudaStream_t s);
 cudaError_t launch_d3q343(Op op, const Args &a, cudaStream_t s);
 
+// Many steps of one D1Q7 tube in one launch: from a.src to a.dst, which may
+// be the same buffer (lbm_d1q7.cu).
+bool tube_steps_ok(const Args &a, int64_t steps);
+cudaError_t launch_tube_steps(const Args &a, int64_t steps, cudaStream_t s);
+
 }  // namespace lbm
