@@ -466,6 +466,8 @@ __global__ void __launch_bounds__(kQ343Block, LBM_Q343_MIN_BLOCKS)
     extern __shared__ unsigned char q343_smem[];
     ST *stash = reinterpret_cast<ST *>(q343_smem);  // [NS planes x 49][kQ343Block] raw values
     constexpr int NS = StashPlanes<ST>::value;
+    pdl_wait();
+    pdl_trigger();
     const Q343Sums s = q343_sums<NS>(p, o, z, stash);
     if constexpr (Q343Dev<ST>::value) q343_collide_dev<ROT, NS>(p, qw, o, z, s, stash);
     else q343_collide<ROT, NS>(p, qw, o, z, s, stash);
@@ -538,8 +540,7 @@ template <bool ROT, typename ST> cudaError_t launch_step_q343(const Args &a, cud
     for (int c = 0; c < 7; ++c) qw.wc[c] = a.wr[c];
     qw.iw_rest = (float)(1.0 / ((double)a.wr[3] * (double)a.wr[3] * (double)a.wr[3]));
     qw.iw_unit = (float)(1.0 / ((double)a.wr[2] * (double)a.wr[3] * (double)a.wr[3]));
-    k_step_q343<ROT, ST><<<grid, kQ343Block, sh, s>>>(p, qw);
-    return cudaGetLastError();
+    return launch_pdl(k_step_q343<ROT, ST>, grid, dim3(kQ343Block), sh, s, p, qw);
 }
 
 cudaError_t launch_d3q343(Op op, const Args &a, cudaStream_t s) { return launch_lattice<4>(op, a, s); }

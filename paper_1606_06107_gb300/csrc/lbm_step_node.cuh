@@ -73,6 +73,8 @@ k_step_node(const Params<Lattice<LAT>::Q, ST> p)
     }
     const uint32_t S = (uint32_t)p.S;
     const int self = oy[3] + ox[3];
+    pdl_wait();
+    pdl_trigger();
 
     // ---- pull the deviations: g_i(x) = ft_i(x - e_i) ----------------------
     float d[Q], h[7];
