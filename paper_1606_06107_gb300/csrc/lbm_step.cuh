@@ -1128,6 +1128,7 @@ __global__ void __launch_bounds__(kBlockX) k_set_state(const Params<Lattice<LAT>
 }
 
 #include "lbm_step_node.cuh"
+#include "lbm_step_pair.cuh"
 
 // ---------------------------------------------------------------------------
 // Host-side dispatch for one lattice.
@@ -1154,6 +1155,15 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// Moments of two nodes per thread (lbm_step_pair.cuh): 16-bit deviations from
+// rest on the 2-D lattices, STREAM transport.
+template <int LAT, int MODE, typename ST> constexpr bool pair_form()
+{
+    return (LAT == 2 || LAT == 3) && MODE == 0 && sizeof(ST) == 2 && !NodeRef<ST>::value;
+}
+// Pairs of an even shift are whole words: no boundary between their columns.
+inline bool pair_whole(const Args &a) { return a.bc[0] == 0 && a.X % 2 == 0; }
+
 // The D3Q343 step (lbm_d3q343.cu): STREAM transport only.
 template <bool ROT, typename ST> cudaError_t launch_step_q343(const Args &a, cudaStream_t s);
 template <bool ROT, typename ST> cudaError_t launch_moments_q343(const Args &a, cudaStream_t s);
@@ -1164,6 +1174,7 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
     const auto p = make_params<Lattice<LAT>::Q, ST>(a);
     const dim3 block(kBlockX);
     const dim3 grid((a.X + kBlockX - 1) / kBlockX, a.Y, a.Z);
+    [[maybe_unused]] const dim3 pairs((a.X + 2 * kBlockX - 1) / (2 * kBlockX), a.Y);
     switch (op) {
     case Op::Step:
         if constexpr (LAT == 4) {  // 343 populations: the two-pass kernel
@@ -1177,7 +1188,10 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
         break;
     case Op::Init: k_init<LAT, ROT, MODE><<<grid, block, 0, s>>>(p); break;
     case Op::Moments:
-        if constexpr (LAT == 4) return launch_moments_q343<ROT, ST>(a, s);
+        if constexpr (pair_form<LAT, MODE, ST>()) {
+            if (pair_whole(a)) k_moments_pair<LAT, ROT, true><<<pairs, block, 0, s>>>(p);
+            else k_moments_pair<LAT, ROT, false><<<pairs, block, 0, s>>>(p);
+        } else if constexpr (LAT == 4) return launch_moments_q343<ROT, ST>(a, s);
         else k_moments<LAT, ROT, MODE><<<grid, block, 0, s>>>(p);
         break;
     case Op::Conserve: k_conserve<LAT, ROT, MODE><<<a.red_blocks, kRedThreads, 0, s>>>(p); break;
