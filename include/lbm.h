@@ -285,10 +285,10 @@ int lbm_batch_bind(lbm_batch b, void *buf_a, void *buf_b, size_t state_bytes, vo
  * the status words.  Asynchronous. */
 int lbm_batch_set_macro(lbm_batch b, const float *rho, const float *u, const float *T);
 
-/* Advance every problem by k >= 0 steps in one persistent launch.  When
- * the longest problem has at most 864 nodes each block holds its problem's
- * two state buffers in shared memory for the whole run (same results, bit
- * for bit).  Asynchronous. */
+/* Advance every problem by k >= 0 steps in one persistent launch.  A problem
+ * of at most 896 nodes stays in a block's shared memory for the whole run, a
+ * longer one goes through it window by window, several steps at a time (same
+ * results, bit for bit).  Asynchronous. */
 int lbm_batch_run(lbm_batch b, int64_t k);
 
 /* rho, u, T of every problem (layout above).  Asynchronous. */
@@ -298,10 +298,10 @@ int lbm_batch_get_moments(lbm_batch b, float *rho, float *u, float *T);
  * and the number of problems whose word is non-zero.  Synchronizing. */
 int lbm_batch_status(lbm_batch b, int *status, int *n_bad);
 
-/* Shape of the persistent launch: threads per block (32..1024, a multiple of
- * 32) and resident blocks per SM (0 = as many as fit; fewer keep more of
- * each problem's state in L2).  lbm_batch_autotune times `sample_steps`
- * steps of the bound ensemble for every pair of 128/256/512/1024 threads and
+/* Shape of the persistent launch: nodes a block updates at a time, two per
+ * thread (`threads`: 32..1024, a multiple of 32), and resident blocks per SM
+ * (0 = as many as fit; fewer keep more of each problem's state in L2).  lbm_batch_autotune times `sample_steps`
+ * steps of the bound ensemble for every pair of 128/256/512/1024 nodes and
  * 1/2/4/max blocks per SM and keeps the fastest (returned through the
  * pointers, which may be NULL).  Autotuning advances the state: call
  * lbm_batch_set_macro afterwards. */

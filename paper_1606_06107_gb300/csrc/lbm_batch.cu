@@ -2,15 +2,10 @@
 // by one persistent launch: the lbm_batch_* part of the C ABI (include/lbm.h).
 //
 // Each resident block claims whole problems, longest first, from an atomic
-// counter and runs all k steps of its problem with a block barrier between
-// steps; the node update is the same device code as lbm_step's (k_step), so
-// results are bit-identical to running each problem alone.  Loads use the
-// L2-coherent path because the launch reads back what it wrote one step
-// earlier.  A problem of L nodes keeps 2 x 14 x L floats live, so the
-// resident problems (a few hundred) stay in the 126 MB L2 for their whole run.
-// When the longest problem has at most 864 nodes, a second form keeps each
-// problem's two buffers in shared memory for the whole run (k_batch_run_sm).
-// A per-problem watch range limits which nodes may set its status word.
+// counter and runs all k steps of its problem; the node update is
+// lbm_step's (lbm_tube.cuh), so results are bit-identical to running each
+// problem alone.  A per-problem watch range limits which nodes may set its
+// status word.
 #include <algorithm>
 #include <cmath>
 #include <numeric>
@@ -20,7 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/lbm.h"
-#include "lbm_step.cuh"
+#include "lbm_tube.cuh"
 
 namespace lbm {
 namespace {
@@ -88,30 +83,49 @@ __device__ __forceinline__ Params<7> tube_params(const BatchParams &bp, const Tu
     return p;
 }
 
-// One node of one problem: the body of k_step<D1Q7, rot, MODE> with
-// L2-coherent loads (CG = 1) or plain loads from shared memory (CG = 2).
-template <int MODE, int CG = 1>
-__device__ __forceinline__ void batch_node(const Params<7> &p, const TubeDesc &d, int x)
-{
-    const Offsets o = node_offsets<1>(p, x, 0, 0);
-    float g[7], h[7];
-    load_node<kD1, true, MODE, CG>(p, o, g, h);
-    const Moments m = node_moments<kD1, true>(p, g, h);
-    if ((!(m.rho > 0.f) || !(m.T > 0.f) || !(fabsf(m.T) < 3.0e38f)) && x >= d.watch_lo &&
-        x < d.watch_hi)
-        atomicOr(p.status, 1);
-    collide_store<kD1>(p, o.self(), g, m, [&](auto ic, float gi) {
-        return transport<kD1, MODE, decltype(ic)::value, CG>(p, o, gi);
-    });
-    float adv[7];
-    rot_advect<1, CG>(p, o, h, m, adv);
-    rot_store(p, o.self(), h, m, adv);
-}
+// The state of the nodes a block works on lies in shared memory, two copies,
+// node by node and 15 floats apart: every population and neighbour is an
+// immediate offset from one address (a third of the instructions of the
+// population-major form were address arithmetic), and the odd pitch keeps
+// consecutive lanes on different banks.  Each thread updates two nodes at a
+// time, half a window apart, in packed arithmetic (f32x2), with a block
+// barrier between steps and three copies of an end's node beyond it.
+//
+// A problem that fits (kWindow nodes, 108 KB: two blocks an SM) is loaded once
+// and stored after its last step.  A longer one goes through the two global
+// buffers in passes of at most kPassSteps steps: a pass loads each window of
+// the problem with as many nodes beside it as the steps can reach (two a step,
+// three in STREAM mode), runs them, and stores the window's inside, which is
+// exactly what whole steps give; the nodes beside it go wrong from the
+// window's ends inwards and are dropped.  Against one pass over the global
+// buffers per step this reads and writes L2 once in sixteen steps, for 8-12 %
+// more nodes.  Bound by shared-memory reads (57 % of the LSU's
+// rate at 1024 windows of 384 nodes) and the barriers between steps: 1024 x
+// 384 nodes, 32 FD steps 180 us (261 with one node per thread, population by
+// population); 1024 tubes of 256-8192 nodes, 50 FD steps 3.43 ms (6.53 through
+// the global buffers).  Passes of 8 / 12 / 16 steps 3.66 / 3.52 / 3.43 ms;
+// windows of 448 nodes 3.84; 256 / 1024 nodes at a time 4.57 / 4.38.
+constexpr int kNodePitch = 15;
+#ifndef LBM_BATCH_WINDOW
+#define LBM_BATCH_WINDOW 896
+#endif
+#ifndef LBM_BATCH_PASS
+#define LBM_BATCH_PASS 16
+#endif
+constexpr int kWindow = LBM_BATCH_WINDOW;
+constexpr int kPassSteps = LBM_BATCH_PASS;
+#ifndef LBM_BATCH_THREADS
+#define LBM_BATCH_THREADS 512
+#endif
 
+// (768: at most 512 threads run; the bound keeps the registers at 80, so that
+// four blocks of 192 threads fit an SM)
 template <int MODE>
-__global__ void __launch_bounds__(1024) k_batch_run(const BatchParams bp)
+__global__ void __launch_bounds__(768) k_batch_run(const BatchParams bp, const TubeLattice lat, int nodes)
 {
+    extern __shared__ float sm[];  // [2][nodes][kNodePitch]
     __shared__ int claim;
+    constexpr int kReach = MODE ? 2 : 3;
     for (;;) {
         if (threadIdx.x == 0) claim = atomicAdd(bp.counter, 1);
         __syncthreads();
@@ -120,55 +134,94 @@ __global__ void __launch_bounds__(1024) k_batch_run(const BatchParams bp)
         if (slot >= bp.count) return;
         const int k = bp.order[slot];
         const TubeDesc d = bp.tubes[k];
+        const TubeRates rates = tube_rates(d.omega, d.cT, d.half_n);
+        // passes: one if the problem fits, else enough of them for the longest
+        // to be kPassSteps and their parity that of the steps, which decides
+        // the buffer the caller expects the state in
+        const bool fits = d.len <= nodes - 6;
+        int64_t passes = 1;
+        if (!fits) {
+            passes = (bp.steps + kPassSteps - 1) / kPassSteps;
+            passes += (passes ^ bp.steps) & 1;
+        }
+        const int halo = fits ? 0 : kReach * kPassSteps;
+        const int windows = fits ? 1 : (d.len + (nodes - 6 - 2 * halo) - 1) / (nodes - 6 - 2 * halo);
         int cur = bp.cur;
-        for (long long s = 0; s < bp.steps; ++s) {
-            Params<7> p = tube_params(bp, d, bp.buf[cur], bp.buf[cur ^ 1]);
-            p.status = bp.status + k;
-            for (int x = threadIdx.x; x < d.len; x += blockDim.x) batch_node<MODE>(p, d, x);
-            cur ^= 1;
-            __syncthreads();  // step s+1 reads neighbours written in step s
+        for (int64_t q = 0; q < passes; ++q) {
+            const int64_t steps = bp.steps * (q + 1) / passes - bp.steps * q / passes;
+            const int end = fits ? bp.cur ^ (int)(bp.steps & 1) : cur ^ 1;
+            const float *in = bp.buf[cur] + d.base;
+            float *out = bp.buf[end] + d.base;
+            for (int wi = 0; wi < windows; ++wi) {
+                const int i0 = (int)((int64_t)d.len * wi / windows), i1 = (int)((int64_t)d.len * (wi + 1) / windows);
+                const int w0 = max(0, i0 - halo), w1 = min(d.len, i1 + halo), n = w1 - w0;
+                float *a = sm, *c = sm + nodes * kNodePitch;
+                // local node l + 3 is node w0 + l; the ends' copies, and
+                // nothing to rely on beyond a window's inner end
+                for (int l = threadIdx.x; l < n + 6; l += blockDim.x) {
+                    const int x = min(max(w0 + l - 3, 0), d.len - 1);
+#pragma unroll
+                    for (int i = 0; i < 14; ++i) a[l * kNodePitch + i] = __ldcg(in + (uint32_t)(i * d.pitch + x));
+                }
+                __syncthreads();
+                const bool left = w0 == 0, right = w1 == d.len;
+                const int half = (n + 1) / 2;
+                for (int64_t s = 0; s < steps; ++s) {
+                    for (int l = threadIdx.x; l < half; l += blockDim.x) {
+                        const bool two = l + half < n;
+                        const int l1 = two ? l + half : l;
+                        const float *m0 = a + (l + 3) * kNodePitch, *m1 = a + (l1 + 3) * kNodePitch;
+                        float *o0 = c + (l + 3) * kNodePitch, *o1 = c + (l1 + 3) * kNodePitch;
+                        F2 rho, T;
+                        tube_update<true, MODE, F2>(
+                            lat, rates,
+                            [&](int pop, int dx) { return f2(m0[dx * kNodePitch + pop], m1[dx * kNodePitch + pop]); },
+                            [&](F2 ux) {
+                                const int p0 = lo(ux) >= 0.f ? -kNodePitch : kNodePitch;
+                                const int p1 = hi(ux) >= 0.f ? -kNodePitch : kNodePitch;
+                                const float *u0 = m0 + p0, *v0 = m0 + 2 * p0, *d0 = m0 - p0;
+                                const float *u1 = m1 + p1, *v1 = m1 + 2 * p1, *d1 = m1 - p1;
+                                return [=](int j, int kk) {
+                                    return kk == 2 ? f2(v0[7 + j], v1[7 + j])
+                                                   : kk == 1 ? f2(u0[7 + j], u1[7 + j]) : f2(d0[7 + j], d1[7 + j]);
+                                };
+                            },
+                            [&](int pop, F2 v) {
+                                o0[pop] = lo(v);
+                                if (two) o1[pop] = hi(v);
+                            },
+                            rho, T);
+                        const int x0 = w0 + l, x1 = w0 + l1;
+                        const int lo_w = max(i0, d.watch_lo), hi_w = min(i1, d.watch_hi);
+                        if ((tube_bad(lo(rho), lo(T)) && x0 >= lo_w && x0 < hi_w) ||
+                            (tube_bad(hi(rho), hi(T)) && x1 >= lo_w && x1 < hi_w))
+                            atomicOr(bp.status + k, 1);
+                        // the copies beyond the problem's ends
+                        if (left && l == 0) {
+#pragma unroll 1
+                            for (int g = 0; g < 3; ++g)
+                                for (int i = 0; i < 14; ++i) c[g * kNodePitch + i] = o0[i];
+                        }
+                        if (right && l1 == n - 1) {
+#pragma unroll 1
+                            for (int g = 0; g < 3; ++g)
+                                for (int i = 0; i < 14; ++i) c[(n + 3 + g) * kNodePitch + i] = o1[i];
+                        }
+                    }
+                    float *t = a;
+                    a = c;
+                    c = t;
+                    __syncthreads();  // step s + 1 reads neighbours written in step s
+                }
+                for (int l = threadIdx.x; l < i1 - i0; l += blockDim.x) {
+#pragma unroll
+                    for (int i = 0; i < 14; ++i)
+                        out[(uint32_t)(i * d.pitch + i0 + l)] = a[(i0 - w0 + l + 3) * kNodePitch + i];
+                }
+                __syncthreads();  // the window's state has been read; its stores precede the next pass
+            }
+            cur = end;
         }
-    }
-}
-
-// The same schedule for problems whose two state buffers fit in shared
-// memory (14 x pitch floats each): the block copies its problem in, steps
-// it between two shared-memory buffers (a step is then bound by shared-
-// memory latency instead of the L2 round trip of each neighbour load), and
-// copies the result to the global buffer the other form would end in.  The
-// node update is the same code, so the results are the same bits.
-template <int MODE>
-__global__ void __launch_bounds__(1024) k_batch_run_sm(const BatchParams bp)
-{
-    extern __shared__ float sm[];
-    __shared__ int claim;
-    for (;;) {
-        if (threadIdx.x == 0) claim = atomicAdd(bp.counter, 1);
-        __syncthreads();
-        const int slot = claim;
-        __syncthreads();  // every thread has read `claim` before it is reused
-        if (slot >= bp.count) return;
-        const int k = bp.order[slot];
-        const TubeDesc d = bp.tubes[k];
-        const int n = 14 * d.pitch;
-        float *a = sm, *c = sm + n;  // a holds the current state
-        const float *in = bp.buf[bp.cur] + d.base;
-        for (int e = threadIdx.x; e < n; e += blockDim.x) a[e] = __ldcg(in + e);
-        __syncthreads();
-        for (long long s = 0; s < bp.steps; ++s) {
-            Params<7> p = tube_params(bp, d, nullptr, nullptr);
-            p.src = a;
-            p.dst = c;
-            p.status = bp.status + k;
-            for (int x = threadIdx.x; x < d.len; x += blockDim.x) batch_node<MODE, 2>(p, d, x);
-            float *t = a;
-            a = c;
-            c = t;
-            __syncthreads();  // step s+1 reads neighbours written in step s
-        }
-        float *out = bp.buf[bp.cur ^ (int)(bp.steps & 1)] + d.base;
-        for (int e = threadIdx.x; e < n; e += blockDim.x) out[e] = a[e];
-        // the claim's barriers order these reads before the next copy-in
     }
 }
 
@@ -209,13 +262,6 @@ void d1q7(double *r, double w[7])
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 
-// Largest shared-memory state (two buffers of the longest problem) for
-// which a run takes the shared-memory form: 96 KB keeps at least two blocks
-// per SM (problems of up to 864 nodes).
-#ifndef LBM_BATCH_SMEM_MAX
-#define LBM_BATCH_SMEM_MAX (96 * 1024)
-#endif
-
 }  // namespace
 }  // namespace lbm
 
@@ -228,7 +274,7 @@ struct lbm_batch_ctx {
     std::vector<TubeDesc> tubes;
     std::vector<int> order;
     int max_len = 0;
-    int sm_bytes = 0;  // > 0: runs take the shared-memory form with this much per block
+    int window = 0;    // nodes a block's shared memory holds, six of them beyond the ends
     int64_t total_nodes = 0;
     size_t state_floats = 0;
     size_t off_tubes = 0, off_order = 0, off_status = 0, off_counter = 0, work_bytes = 0;
@@ -237,8 +283,8 @@ struct lbm_batch_ctx {
     char *work = nullptr;
     cudaStream_t stream = nullptr;
     int cur = 0;
-    int threads = 256;
-    int blocks_per_sm = 0;  // resident blocks per SM of the persistent grid (0 = max)
+    int threads = LBM_BATCH_THREADS;  // nodes a block updates at a time, two a thread
+    int blocks_per_sm = 0;            // resident blocks per SM of the persistent grid (0 = max)
     int64_t launches = 0;
     std::string err;
     struct Cached {
@@ -289,16 +335,14 @@ BatchParams batch_params(const lbm_batch_ctx *b, long long steps)
 
 bool aligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
 
-// The persistent kernel of a run: the shared-memory form when the longest
-// problem fits (sm_bytes > 0), else the global-memory form.
+// The persistent kernel of a run, its threads (two nodes each) and its
+// dynamic shared memory.
 const void *run_kernel(const lbm_batch_ctx *b)
 {
-    if (b->sm_bytes > 0)
-        return (b->mode == LBM_MODE_FD) ? (const void *)lbm::k_batch_run_sm<1>
-                                        : (const void *)lbm::k_batch_run_sm<0>;
-    return (b->mode == LBM_MODE_FD) ? (const void *)lbm::k_batch_run<1>
-                                    : (const void *)lbm::k_batch_run<0>;
+    return (b->mode == LBM_MODE_FD) ? (const void *)lbm::k_batch_run<1> : (const void *)lbm::k_batch_run<0>;
 }
+int run_threads(int threads) { return std::max(32, (threads / 2 + 31) / 32 * 32); }
+int run_smem(const lbm_batch_ctx *b) { return (int)sizeof(float) * 2 * lbm::kNodePitch * b->window; }
 
 // Resident-block grid of the persistent kernel for `threads` per block.
 cudaError_t persistent_grid(const lbm_batch_ctx *b, int threads, int bps, int *grid)
@@ -308,10 +352,14 @@ cudaError_t persistent_grid(const lbm_batch_ctx *b, int threads, int bps, int *g
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const void *fn = run_kernel(b);
-    if (b->sm_bytes > 0)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, b->sm_bytes);
+    // (the limit is a property of the kernel, which other ensembles share: the
+    // largest any of them takes)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(float) * 2 * lbm::kNodePitch * (lbm::kWindow + 6));
+    if (e == cudaSuccess)  // all of L1 as shared memory: the kernel reads nothing twice through it
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, b->sm_bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, run_threads(threads), run_smem(b));
     if (e != cudaSuccess) return e;
     per_sm = std::max(1, per_sm);
     if (bps > 0) per_sm = std::min(per_sm, bps);
@@ -338,12 +386,14 @@ int build_graph(lbm_batch b, long long steps, cudaGraphExec_t *exec)
     cudaGraphNode_t n_reset = nullptr, n_run = nullptr;
     e = cudaGraphAddMemsetNode(&n_reset, g, nullptr, 0, &ms);
     BatchParams bp = batch_params(b, steps);
-    void *args[] = {&bp};
+    lbm::TubeLattice lat = lbm::tube_lattice(bp.w, bp.r, bp.nu_scale, bp.inv_m);
+    int window = b->window;
+    void *args[] = {&bp, &lat, &window};
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void *>(run_kernel(b));
     kp.gridDim = dim3(grid);
-    kp.blockDim = dim3(b->threads);
-    kp.sharedMemBytes = (unsigned)b->sm_bytes;
+    kp.blockDim = dim3(run_threads(b->threads));
+    kp.sharedMemBytes = (unsigned)run_smem(b);
     kp.kernelParams = args;
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&n_run, g, &n_reset, 1, &kp);
     if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
@@ -403,8 +453,7 @@ int lbm_batch_create(int count, const int64_t *lengths, const int *n, const doub
     }
     b->state_floats = base;
     b->total_nodes = node;
-    const size_t sm = (size_t)2 * 14 * ((b->max_len + 31) / 32 * 32) * sizeof(float);
-    b->sm_bytes = (sm <= (size_t)LBM_BATCH_SMEM_MAX) ? (int)sm : 0;
+    b->window = std::min(b->max_len, lbm::kWindow) + 6;
     b->order.resize(count);
     std::iota(b->order.begin(), b->order.end(), 0);
     std::stable_sort(b->order.begin(), b->order.end(),

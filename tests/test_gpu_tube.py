@@ -67,3 +67,33 @@ def test_captured_steps(kind, shape, storage):
         torch.cuda.synchronize()
         for x, y in zip(sims[0].moments(), sims[1].moments()):
             assert bool(torch.isfinite(x).all()) and torch.equal(x, y)
+
+
+@pytest.mark.parametrize("mode", ["fd", "stream"])
+@pytest.mark.parametrize("block", [32, 96, 512, 1024])
+def test_windowed_ensemble_equals_single_runs(mode, block):
+    """Tubes around the window's size and several windows long, for step
+    counts around a pass and of both parities, with a block of one warp and
+    of more threads than a short tube has nodes."""
+    from paper_1606_06107_gb300 import Lbm, LbmBatch
+    lengths = [1, 2, 3, 63, 895, 896, 897, 1337, 1745, 5000]
+    ns = [0, 2, 4, 6, 7, 2, 4, 6, 7, 4]
+    wl = [workloads.smooth_random((L,), seed=L, kind="D1Q7", n=4, u_mean=[0.1]) for L in lengths]
+    cat = [np.concatenate([np.asarray(getattr(w, f)).reshape(-1) for w in wl]) for f in ("rho", "u", "T")]
+    ens = LbmBatch(lengths, ns, [0.8] * len(lengths), mode=mode)
+    ens.set_block(block)
+    sims = [Lbm("D1Q7", n, 0.8, (L,), ("copy",), mode=mode) for L, n in zip(lengths, ns)]
+    for steps in ([1, 2, 7, 8], [9, 16], [33]):
+        ens.set_macro(*cat)
+        for s, w in zip(sims, wl):
+            s.set_macro(w.rho, w.u, w.T)
+        for k in steps:
+            ens.run(k)
+            for s in sims:
+                s.step(k)
+        got = [x.cpu().numpy() for x in ens.moments()]
+        for k, s in enumerate(sims):
+            sl = slice(ens.offsets[k], ens.offsets[k] + lengths[k])
+            for a, b in zip(got, s.moments()):
+                assert np.array_equal(a[sl], b.cpu().numpy().reshape(-1)), (k, steps)
+    assert ens.status()[1] == 0
