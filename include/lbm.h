@@ -369,6 +369,11 @@ int lbm_nn_conv_backward_data(const void *gz, const void *wt, float *gx, const v
 int lbm_nn_conv_backward_weight(const void *gz, const void *x, float *gw, int B, int L, int C, int k,
                                 int dil, int impl, int *status, void *stream);
 
+/* The same and, if gb is not NULL, the bias gradient in the same pass:
+ * gb[co] += sum_{b,l} gz[b,l,co] (as lbm_nn_bias_grad). */
+int lbm_nn_conv_backward_weight_bias(const void *gz, const void *x, float *gw, float *gb, int B, int L,
+                                     int C, int k, int dil, int impl, int *status, void *stream);
+
 /* bf16 copies of `layers` float conv weights [layers][k][C][C]: w_bf16 in
  * the same layout, wt_bf16 (may be NULL) transposed and flipped per layer. */
 int lbm_nn_cast_weights(const float *w, void *w_bf16, void *wt_bf16, int layers, int C, int k,

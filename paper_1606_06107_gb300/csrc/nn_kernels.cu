@@ -311,12 +311,13 @@ __device__ __forceinline__ Smem carve(uint8_t *raw)
     return s;
 }
 
-__device__ __forceinline__ void setup(const Smem &s)
+// `readers`: arrivals that free a stage (the MMAs' commit, and warps that read it).
+__device__ __forceinline__ void setup(const Smem &s, int readers = 1)
 {
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
             mbar_init(&s.full[i], 1);
-            mbar_init(&s.empty[i], 1);
+            mbar_init(&s.empty[i], readers);
         }
         mbar_init(s.done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -881,9 +882,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
 // Weight gradient: one block reduces the positions of blocks [q0, q1) (64
 // positions each, tubes one after another) for one tap and one 128 x 128
 // (co, ci) tile, then adds its tile to gw with coalesced vector reductions.
+// With gb, the two warps that neither load nor issue add up the columns of the
+// g_z tiles of the first tap and first ci tile, which pass through shared
+// memory anyway: the bias gradient (6.5 us a layer as a kernel of its own at
+// 2^15 positions).
 __global__ void __launch_bounds__(128, 1)
     k_wgrad_tc(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_x,
-               float *gw, int B, int L, int C, int k, int dil, int per_block, int *status)
+               float *gw, float *gb, int B, int L, int C, int k, int dil, int per_block, int *status)
 {
     extern __shared__ uint8_t smem_raw[];
     const Smem s = carve(smem_raw);
@@ -896,7 +901,8 @@ __global__ void __launch_bounds__(128, 1)
     const int q0 = blockIdx.x * per_block, q1 = std::min(total, q0 + per_block);
     if (q0 >= q1) return;  // uniform across the block, before any allocation
     const int nk = q1 - q0, shift = (t - k / 2) * dil;
-    setup(s);
+    const bool columns = gb && t == 0 && ci0 == 0;
+    setup(s, columns ? 3 : 1);
     const uint32_t tmem = *s.tmem_slot;
     __shared__ volatile int failed;
     if (threadIdx.x == 0) failed = 0;
@@ -941,12 +947,44 @@ __global__ void __launch_bounds__(128, 1)
             mma_commit(&s.empty[st]);
         }
         mma_commit(s.done);
+    } else if (warp >= 2 && columns) {
+        // channels co0 + 2 v and the next: 32 lanes cover one 128-byte row of a
+        // 64-channel block, whose 16-byte chunks lie at (chunk ^ row % 8)
+        const int v = (warp - 2) * 32 + lane, chunk = (v & 31) >> 2;
+        float s0 = 0.f, s1 = 0.f;
+        bool ok = true;
+        for (int kb = 0; kb < nk; ++kb) {
+            const int st = kb % kStages;
+            if (!mbar_wait(&s.full[st], (kb / kStages) & 1, status)) {
+                failed = 1;
+                ok = false;
+                break;
+            }
+            const uint8_t *box = s.tiles + st * kStageBytes + (v >> 5) * 8192 + (v & 3) * 4;
+            float t0 = 0.f, t1 = 0.f;
+#pragma unroll 16
+            for (int r = 0; r < kWgRows; ++r) {
+                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(
+                    box + r * 128 + ((chunk ^ (r & 7)) << 4)));
+                t0 += f.x;
+                t1 += f.y;
+            }
+            s0 += t0;
+            s1 += t1;
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&s.empty[st])) : "memory");
+        }
+        if (ok) {
+            atomicAdd(gb + co0 + 2 * v, s0);
+            atomicAdd(gb + co0 + 2 * v + 1, s1);
+        }
     }
     __syncwarp();
     if (!mbar_wait(s.done, 0, status)) failed = 1;
     __syncwarp();
     tc_fence_after();
 
+    if (columns) __syncthreads();  // the column sums have read the last tiles
     // stage 32 x 32 blocks through shared memory (the pipeline buffers are
     // free once the last MMA has completed) so that a warp adds 32
     // consecutive columns of one row at a time
@@ -1962,9 +2000,19 @@ int lbm_nn_conv_backward_data(const void *gz, const void *wt, float *gx, const v
 int lbm_nn_conv_backward_weight(const void *gz, const void *x, float *gw, int B, int L, int C, int k,
                                 int dil, int impl, int *status, void *stream)
 {
+    return lbm_nn_conv_backward_weight_bias(gz, x, gw, nullptr, B, L, C, k, dil, impl, status, stream);
+}
+
+int lbm_nn_conv_backward_weight_bias(const void *gz, const void *x, float *gw, float *gb, int B, int L, int C,
+                                     int k, int dil, int impl, int *status, void *stream)
+{
     if (!gz || !x || !gw || !conv_shape_ok(B, L, C, k, dil, impl)) return LBM_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     if (impl == 1) {
+        if (gb) {
+            const int rc = lbm_nn_bias_grad(gz, gb, (int64_t)B * L, C, stream);
+            if (rc != LBM_OK) return rc;
+        }
         const dim3 grid((L + kSimtTX - 1) / kSimtTX, (C / kSimtTC) * (C / kSimtCI), B);
         k_wgrad_simt<<<grid, 256, 0, s>>>((const __nv_bfloat16 *)gz, (const __nv_bfloat16 *)x, gw,
                                           L, C, k, dil);
@@ -1977,11 +2025,14 @@ int lbm_nn_conv_backward_weight(const void *gz, const void *x, float *gw, int B,
     if (!map_act(&mg, gz, B, L, C, kWgRows) || !map_act(&mx, x, B, L, C, kWgRows)) return LBM_ECUDA;
     const int tiles = (C / kTile) * (C / kTile) * k;
     const int64_t total = (int64_t)B * ((L + kWgRows - 1) / kWgRows);
+#ifndef LBM_WGRAD_PER_SM
+#define LBM_WGRAD_PER_SM 2
+#endif
     // about two resident blocks per SM in one wave
-    const int64_t want = std::max<int64_t>(1, (2 * 152 + tiles - 1) / tiles);
+    const int64_t want = std::max<int64_t>(1, (LBM_WGRAD_PER_SM * 152 + tiles - 1) / tiles);
     const int per_block = (int)std::max<int64_t>(1, (total + want - 1) / want);
     const int chunks = (int)((total + per_block - 1) / per_block);
-    k_wgrad_tc<<<dim3(chunks, tiles), 128, kSmemBytes, s>>>(mg, mx, gw, B, L, C, k, dil, per_block,
+    k_wgrad_tc<<<dim3(chunks, tiles), 128, kSmemBytes, s>>>(mg, mx, gw, gb, B, L, C, k, dil, per_block,
                                                             status);
     return launched(cudaGetLastError());
 }

@@ -83,6 +83,8 @@ SIGNATURES = {
                                   + [_vp, _vp]),
     "lbm_nn_conv_backward_weight": (ctypes.c_int, [_vp, _vp, _vp] + [ctypes.c_int] * 6
                                     + [_vp, _vp]),
+    "lbm_nn_conv_backward_weight_bias": (ctypes.c_int, [_vp, _vp, _vp, _vp] + [ctypes.c_int] * 6
+                                         + [_vp, _vp]),
     "lbm_nn_cast_weights": (ctypes.c_int, [_vp, _vp, _vp, ctypes.c_int, ctypes.c_int,
                                            ctypes.c_int, _vp]),
     "lbm_nn_lift": (ctypes.c_int, [_vp, _vp, _vp, _vp, _i64, ctypes.c_int, ctypes.c_int, _vp]),

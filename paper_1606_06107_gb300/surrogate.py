@@ -220,12 +220,12 @@ class ConvOperator:
         cur = 0
         for i in reversed(range(self.N)):
             d = self.dil[i]
-            self._check(lib.lbm_nn_bias_grad(_fp(gz[cur]), self._ptr(g, "b", i), P, self.C, s),
-                        "lbm_nn_bias_grad")
-            self._check(lib.lbm_nn_conv_backward_weight(_fp(gz[cur]), _fp(x[i]), self._ptr(g, "W", i),
-                                                        B, Lp, self.C, self.k, d,
-                                                        self.conv_impl(d), _fp(self.status), s),
-                        "lbm_nn_conv_backward_weight")
+            self._check(lib.lbm_nn_conv_backward_weight_bias(_fp(gz[cur]), _fp(x[i]),
+                                                             self._ptr(g, "W", i),
+                                                             self._ptr(g, "b", i), B, Lp, self.C,
+                                                             self.k, d, self.conv_impl(d),
+                                                             _fp(self.status), s),
+                        "lbm_nn_conv_backward_weight_bias")
             zp, gzp = (z[i - 1], gz[1 - cur]) if i > 0 else (None, None)
             self._check(lib.lbm_nn_conv_backward_data(_fp(gz[cur]), self._wt(i), _fp(gx), _fp(zp),
                                                       _fp(gzp), B, Lp, self.C, self.k, d,

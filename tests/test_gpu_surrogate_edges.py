@@ -5,7 +5,8 @@ counts off the vector path; tensors off the vectors' alignment.
 
 Tolerances: float32 products and sums, 1e-5 of the sum of the terms'
 magnitudes (a few thousand terms at unit roundoff 6e-8, summed in blocks);
-bfloat16 results half an ulp (2^-9) more, and 2^-10 for the hardware tanh."""
+bfloat16 results 2^-9 of a scale about twice the value's or more (half an ulp
+is at most 2^-8 of the value), and 2^-10 of it for the hardware tanh."""
 import numpy as np
 import pytest
 
@@ -86,6 +87,52 @@ def test_bias_gradient(lib, P, C, skip):
     before = gb.double()
     assert lib.lbm_nn_bias_grad(gz.data_ptr(), gb.data_ptr(), P, C, None) == 0
     close(gb, before + gz.double().sum(0), before.abs() + gz.double().abs().sum(0))
+
+
+@pytest.mark.parametrize("impl", [0, 1, 2, 3])
+@pytest.mark.parametrize("B,L,C,k,d", [(3, 300, 128, 5, 3), (1, 64, 128, 3, 1), (2, 77, 256, 3, 2), (40, 130, 128, 5, 1)])
+def test_bias_gradient_with_the_weight_gradient(lib, impl, B, L, C, k, d):
+    """Both gradients of the joint entry; the bias sums over a few thousand
+    terms in blocks of 64, the weight gradient as its own entry gives it."""
+    import torch
+    gz, x = make(1, B * L, C, dtype="bfloat16"), make(2, B * L, C, dtype="bfloat16")
+    gw, gw2, gb = torch.zeros(k, C, C, device="cuda"), torch.zeros(k, C, C, device="cuda"), make(3, C)
+    before = gb.double()
+    st = torch.zeros(1, device="cuda", dtype=torch.int32)
+    assert lib.lbm_nn_conv_backward_weight_bias(gz.data_ptr(), x.data_ptr(), gw.data_ptr(), gb.data_ptr(), B, L, C, k, d,
+                                                impl, st.data_ptr(), None) == 0
+    assert lib.lbm_nn_conv_backward_weight(gz.data_ptr(), x.data_ptr(), gw2.data_ptr(), B, L, C, k, d, impl, st.data_ptr(),
+                                           None) == 0
+    assert int(st) == 0
+    close(gb, before + gz.double().sum(0), before.abs() + gz.double().abs().sum(0))
+    close(gw, gw2.double(), (gz.double().abs().T @ x.double().abs())[None].expand(k, -1, -1))
+
+
+@pytest.mark.parametrize("B,L,skip", [(1, 1, 0), (3, 7, 0), (5, 12, 0), (255, 4112, 0), (256, 4096, 0),
+                                      (256, 4096, 1), (1051, 1001, 0), (1051, 1004, 0)])
+def test_features_targets_and_update(lib, B, L, skip):
+    import ctypes
+    import torch
+    n = B * L
+    a, b = [make(k, n, skip=skip) for k in (1, 2, 3)], [make(k, n, skip=skip) for k in (4, 5, 6)]
+    gamma, out = make(7, B), make(8, 3 * n, skip=skip)
+    feat, tgt = torch.empty(n, 4, device="cuda"), make(9, 3 * n, skip=skip)
+    new = [make(9 + k, n, skip=skip) for k in (1, 2, 3)]
+    s4, s3 = (ctypes.c_float * 4)(1.0, 0.5, 2.0, 0.25), (ctypes.c_float * 3)(0.05, 0.04, 0.06)
+    ptr = lambda v: [x.data_ptr() for x in v]  # noqa: E731
+    assert lib.lbm_nn_features(*ptr(a), gamma.data_ptr(), feat.data_ptr(), B, L, s4, None) == 0
+    assert lib.lbm_nn_targets(*ptr(a), *ptr(b), tgt.data_ptr(), n, s3, None) == 0
+    assert lib.lbm_nn_apply(*ptr(a), out.data_ptr(), *ptr(new), n, s3, None) == 0
+    da, db = [v.double() for v in a], [v.double() for v in b]
+    g = torch.repeat_interleave(gamma.double(), L)
+    want = torch.stack([(da[0] - 1), da[1] / 0.5, (da[2] - 1) / 2, (g - 1.4) / 0.25], 1)
+    close(feat, want, 10 * (1 + want.abs()), rel=1e-6)
+    scale = torch.tensor([np.float32(v) for v in (0.05, 0.04, 0.06)], device="cuda", dtype=torch.float64)
+    want = torch.stack([y - x for x, y in zip(da, db)], 1) / scale
+    close(tgt.view(n, 3), want, want.abs() + 100, rel=1e-6)
+    for k in range(3):
+        want = da[k] + out.double().view(n, 3)[:, k] * scale[k]
+        close(new[k], want, da[k].abs() + 1, rel=1e-6)
 
 
 @pytest.mark.parametrize("n", [1, 255, 257, 311297])
