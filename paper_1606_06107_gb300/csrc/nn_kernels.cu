@@ -266,6 +266,25 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 lanes x 16 consecutive fp32 columns of the accumulator.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+        "%12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+                   "+r"(r[14]), "+r"(r[15])
+                 :: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // ------------------------------------------------------------ GEMM kernels
 enum Epi : int { kEpiForward = 0, kEpiInputGrad = 1 };
 
@@ -473,7 +492,7 @@ constexpr int kPSmemBytes = kPStages * kStageBytes + kStagingBytes + 1024 + 256;
 // through a padded shared-memory block (pitch COLS + 4 floats) so that every
 // global load and store is done cooperatively: COLS/4 lanes cover the COLS
 // columns of one row, so each instruction touches whole row segments.
-template <int EPI, int COLS = 64>
+template <int EPI, int COLS = 64, int ROWS = 32>
 __device__ __forceinline__ void finish_rows(const ConvArgs &a, const float *st, int b, int l_first,
                                             int n0, bool skip);
 
@@ -497,11 +516,11 @@ __device__ __forceinline__ void epilogue_rows(const ConvArgs &a, float *st, uint
     finish_rows<EPI, COLS>(a, st, b, l_first, n0, skip);
 }
 
-// Second half of the epilogue: the staged block (32 rows = positions
+// Second half of the epilogue: the staged block (ROWS rows = positions
 // l_first.., COLS channels n0.., pitch COLS + 4 floats) is read back so
 // that COLS/4 lanes cover the COLS channels of one row and every global
 // load and store touches whole row segments.
-template <int EPI, int COLS>
+template <int EPI, int COLS, int ROWS>
 __device__ __forceinline__ void finish_rows(const ConvArgs &a, const float *st, int b, int l_first,
                                             int n0, bool skip)
 {
@@ -515,7 +534,7 @@ __device__ __forceinline__ void finish_rows(const ConvArgs &a, const float *st, 
         // kBatch: all loads of a group are issued before any result is formed
         const int64_t row0 = ((int64_t)b * a.L + l_first) * a.C + n0 + cg;
 #pragma unroll 1
-        for (int r0 = lane / kLpr; r0 < 32; r0 += kBatch * kRpi) {
+        for (int r0 = lane / kLpr; r0 < ROWS; r0 += kBatch * kRpi) {
             float4 acc[kBatch], gin[kBatch];
             uint2 in[kBatch];
             bool live[kBatch];
@@ -716,15 +735,23 @@ __global__ void __launch_bounds__(kPThreads, 1)
 // and the k taps read it at row offsets t dil (sub-window descriptors),
 // instead of one shifted tile per tap; the weight tiles stream through a
 // 4-stage ring.  Two 256-column accumulators fill the 512 columns of tensor
-// memory.  After tcgen05.ld a lane holds one channel at 32 positions; the
+// memory.  After tcgen05.ld a lane holds one channel at 16 positions; the
 // staging store writes it transposed, so the read-back and the global I/O
-// are those of the other persistent form.
+// are those of the other persistent form.  Sixteen positions at a time halve
+// the staging memory (37 KB): what the block does not take of the SM's 256 KB
+// caches the epilogue's operands.  2^20 positions, 128 channels, 5 taps: input
+// gradient 338 -> 288 us, forward 167 as before; 2^15 positions 14.5 -> 12.6
+// and 12.6 -> 11.2 us.  A third activation window instead: 334 / 170; the next
+// tile's windows prefetched to L2: 301 / 173; the weights as the MMA's A
+// operand in tensor memory, 96 positions per tile: 374 / 222.
 constexpr int kNPos = 256;                         // positions per tile (MMA N)
 constexpr int kXStages = 2;                        // activation windows in flight
 constexpr int kWStages = 4;                        // weight tiles in flight
+constexpr int kNStageRows = 16;                    // positions a warp stages at a time
+constexpr int kNStagingBytes = kEpiWarps * kNStageRows * kStagePitch * 4;
 constexpr int kWTileBytes = kTile * kChunk * 2;    // 128 channels x 64 input channels
 constexpr int kMaxHalo = 64;                       // largest (k-1) dil a window holds
-constexpr int kNSmemFixed = kWStages * kWTileBytes + kStagingBytes + 1024 + 256;
+constexpr int kNSmemFixed = kWStages * kWTileBytes + kNStagingBytes + 1024 + 256;
 
 // Window rows: 256 + (k-1) dil rounded up to 16, loaded as two boxes of
 // half that (each a multiple of 8 rows, so both halves start 1024-byte aligned).
@@ -754,7 +781,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     uint8_t *xbuf = wbuf + kWStages * kWTileBytes;
     const int xbytes = rows * 128;
     float *staging = (float *)(xbuf + kXStages * xbytes);
-    uint64_t *wfull = (uint64_t *)((uint8_t *)staging + kStagingBytes);
+    uint64_t *wfull = (uint64_t *)((uint8_t *)staging + kNStagingBytes);
     uint64_t *wempty = wfull + kWStages;
     uint64_t *xfull = wempty + kWStages;
     uint64_t *xempty = xfull + kXStages;
@@ -876,7 +903,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         }
     } else {  // epilogue warps: lane quarter warp % 4 (32 channels), 64 positions each
         const int e = warp - 2, quarter = warp & 3, pos0 = (e >> 2) * 64;
-        float *st = staging + e * 32 * kStagePitch;
+        float *st = staging + e * kNStageRows * kStagePitch;
         int it = 0;
         for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++it) {
             const int acc = it & 1, use = it >> 1;
@@ -887,14 +914,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
             if (!ready) failed = 1;
             tc_fence_after();
 #pragma unroll 1
-            for (int h = 0; h < 64; h += 32) {
-                float v[32];
+            for (int h = 0; h < 64; h += kNStageRows) {
+                float v[kNStageRows];
                 __syncwarp();
-                tmem_ld32(tmem + acc * kNPos + ((uint32_t)(quarter * 32) << 16) + pos0 + h, v);
+                tmem_ld16(tmem + acc * kNPos + ((uint32_t)(quarter * 32) << 16) + pos0 + h, v);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) st[j * kStagePitch + lane] = v[j];
+                for (int j = 0; j < kNStageRows; ++j) st[j * kStagePitch + lane] = v[j];
                 __syncwarp();
-                finish_rows<EPI, 32>(a, st, b, l0 + pos0 + h, co0 + quarter * 32, failed != 0);
+                finish_rows<EPI, 32, kNStageRows>(a, st, b, l0 + pos0 + h, co0 + quarter * 32, failed != 0);
             }
             tc_fence_before();
             __syncwarp();
