@@ -487,116 +487,205 @@ constexpr int kStagePitch = 36;  // floats per staged row (32 + 4: conflict-free
 constexpr int kStagingBytes = kEpiWarps * 32 * kStagePitch * 4;
 constexpr int kPSmemBytes = kPStages * kStageBytes + kStagingBytes + 1024 + 256;
 
-// Epilogue of one warp's 32 rows x COLS columns (32 or 64) of a persistent
-// tile.  The accumulator rows (one per lane after tcgen05.ld) are transposed
-// through a padded shared-memory block (pitch COLS + 4 floats) so that every
-// global load and store is done cooperatively: COLS/4 lanes cover the COLS
-// columns of one row, so each instruction touches whole row segments.
-template <int EPI, int COLS = 64, int ROWS = 32>
-__device__ __forceinline__ void finish_rows(const ConvArgs &a, const float *st, int b, int l_first,
-                                            int n0, bool skip);
-
-template <int EPI, int COLS = 64>
-__device__ __forceinline__ void epilogue_rows(const ConvArgs &a, float *st, uint32_t taddr, int b,
-                                              int l_first, int n0, bool skip)
+// Two floats in a register pair: one packed operation in place of two, the
+// same rounding.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
 {
-    constexpr int kPitch = COLS + 4;
-    const int lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int c = 0; c < COLS; c += 32) {
-        float v[32];
-        __syncwarp();
-        tmem_ld32(taddr + c, v);
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// gelu() of two values.
+__device__ __forceinline__ uint64_t gelu2(uint64_t x)
+{
+    const float c = 0.7978845608028654f;
+    float u0, u1;
+    unpack2(mul2(x, fma2(mul2(x, x), pack2(0.044715f * c, 0.044715f * c), pack2(c, c))), u0, u1);
+    const uint64_t h = mul2(pack2(0.5f, 0.5f), x);
+    return fma2(h, pack2(tanh_fast(u0), tanh_fast(u1)), h);
+}
+__device__ __forceinline__ uint4 pack8(const uint64_t *v)
+{
+    uint4 q;
+    __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(&q);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4 *>(st + lane * kPitch + c + 4 * j) =
-                make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    for (int i = 0; i < 4; ++i) {
+        float a, b;
+        unpack2(v[i], a, b);
+        h[i] = __floats2bfloat162_rn(a, b);
     }
-    __syncwarp();
-    finish_rows<EPI, COLS>(a, st, b, l_first, n0, skip);
+    return q;
 }
 
 // Second half of the epilogue: the staged block (ROWS rows = positions
-// l_first.., COLS channels n0.., pitch COLS + 4 floats) is read back so
-// that COLS/4 lanes cover the COLS channels of one row and every global
-// load and store touches whole row segments.
-template <int EPI, int COLS, int ROWS>
+// l_first.., 32 channels n0.., pitch 36 floats) is read back so that four or
+// eight lanes cover the 32 channels of a row and every
+// global access is part of a whole row segment.  All rows' loads are issued
+// before any result is formed.  This is what bounds the inference product: with
+// four channels a lane, 8-byte accesses and scalar arithmetic it takes 22
+// instructions per element, and without it the product runs in 124 us instead
+// of 155 (2^20 positions, 128 channels, 5 taps; the MMAs and loads alone in
+// 99).  Without a pre-activation output a lane therefore takes eight channels
+// in packed arithmetic and 16-byte accesses: 138 us, the same bits.  With it,
+// and in the input gradient, the bytes bound the product (165 and 288 us) and
+// four channels a lane are as fast or faster (eight: 167 and 294; at 2^15
+// positions 11.2 against 11.5 and 12.7 against 14.4).
+template <int EPI, int ROWS>
 __device__ __forceinline__ void finish_rows(const ConvArgs &a, const float *st, int b, int l_first,
                                             int n0, bool skip)
 {
-    constexpr int kPitch = COLS + 4, kLpr = COLS / 4, kRpi = 32 / kLpr, kBatch = 4;
     const int lane = threadIdx.x & 31;
     if (!skip) {
-        const int cg = (lane % kLpr) * 4;
-        float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (EPI == kEpiForward) bias = *reinterpret_cast<const float4 *>(a.bias + n0 + cg);
-        // 32 / kRpi rows per lane (r = lane / kLpr + kRpi i) in groups of
-        // kBatch: all loads of a group are issued before any result is formed
-        const int64_t row0 = ((int64_t)b * a.L + l_first) * a.C + n0 + cg;
-#pragma unroll 1
-        for (int r0 = lane / kLpr; r0 < ROWS; r0 += kBatch * kRpi) {
-            float4 acc[kBatch], gin[kBatch];
-            uint2 in[kBatch];
-            bool live[kBatch];
+        if (EPI == kEpiForward && !a.z) {
+            constexpr int kN = ROWS / 8;  // rows of a lane
+            const int cg = (lane & 3) * 8, r0 = lane >> 2;
+            const int64_t row0 = ((int64_t)b * a.L + l_first + r0) * a.C + n0 + cg;
+            const float *sr = st + r0 * kStagePitch + cg;
+            bool live[kN];
 #pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
-                const int r = r0 + kRpi * i, l = l_first + r;
-                live[i] = l < a.L;
-                acc[i] = *reinterpret_cast<const float4 *>(st + r * kPitch + cg);
-                if (live[i]) {
-                    const int64_t o = row0 + (int64_t)(r * a.C);
-                    if constexpr (EPI == kEpiForward) {
-                        in[i] = *reinterpret_cast<const uint2 *>(a.x + o);
-                    } else {
-                        gin[i] = *reinterpret_cast<const float4 *>(a.gx + o);
-                        if (a.gzprev) in[i] = *reinterpret_cast<const uint2 *>(a.zprev + o);
-                    }
-                }
+            for (int i = 0; i < kN; ++i) live[i] = l_first + r0 + 8 * i < a.L;
+            uint4 in[kN];
+#pragma unroll
+            for (int i = 0; i < kN; ++i)
+                if (live[i]) in[i] = *reinterpret_cast<const uint4 *>(a.x + row0 + (int64_t)(8 * i * a.C));
+            uint64_t bias[4];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(a.bias + n0 + cg) + q);
+                bias[2 * q] = pack2(v.x, v.y);
+                bias[2 * q + 1] = pack2(v.z, v.w);
             }
 #pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
+            for (int i = 0; i < kN; ++i) {
                 if (!live[i]) continue;
-                const int64_t o = row0 + (int64_t)((r0 + kRpi * i) * a.C);
-                if constexpr (EPI == kEpiForward) {
-                    const float2 x01 =
-                        __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&in[i].x));
-                    const float2 x23 =
-                        __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&in[i].y));
-                    const float z0 = acc[i].x + bias.x, z1 = acc[i].y + bias.y,
-                                z2 = acc[i].z + bias.z, z3 = acc[i].w + bias.w;
-                    uint2 yv;
-                    *reinterpret_cast<__nv_bfloat162 *>(&yv.x) =
-                        __floats2bfloat162_rn(x01.x + gelu(z0), x01.y + gelu(z1));
-                    *reinterpret_cast<__nv_bfloat162 *>(&yv.y) =
-                        __floats2bfloat162_rn(x23.x + gelu(z2), x23.y + gelu(z3));
-                    *reinterpret_cast<uint2 *>(a.y + o) = yv;
-                    if (a.z) {
-                        uint2 zv;
-                        *reinterpret_cast<__nv_bfloat162 *>(&zv.x) = __floats2bfloat162_rn(z0, z1);
-                        *reinterpret_cast<__nv_bfloat162 *>(&zv.y) = __floats2bfloat162_rn(z2, z3);
-                        *reinterpret_cast<uint2 *>(a.z + o) = zv;
+                const int64_t o = row0 + (int64_t)(8 * i * a.C);
+                const float4 v0 = *reinterpret_cast<const float4 *>(sr + 8 * i * kStagePitch);
+                const float4 v1 = *reinterpret_cast<const float4 *>(sr + 8 * i * kStagePitch + 4);
+                const uint64_t acc[4] = {pack2(v0.x, v0.y), pack2(v0.z, v0.w), pack2(v1.x, v1.y), pack2(v1.z, v1.w)};
+                float x[8];
+                unpack8(in[i], x);
+                uint64_t y[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    y[q] = add2(pack2(x[2 * q], x[2 * q + 1]), gelu2(add2(acc[q], bias[q])));
+                *reinterpret_cast<uint4 *>(a.y + o) = pack8(y);
+            }
+        } else {
+            // four channels a lane
+            constexpr int kLpr = 8, kRpi = 4, kBatch = 4;
+            static_assert(ROWS % (kBatch * kRpi) == 0, "whole batches");
+            const int cg = (lane % kLpr) * 4;
+            float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (EPI == kEpiForward) bias = *reinterpret_cast<const float4 *>(a.bias + n0 + cg);
+            // 32 / kRpi rows per lane (r = lane / kLpr + kRpi i) in groups of
+            // kBatch: all loads of a group are issued before any result is formed
+            const int64_t row0 = ((int64_t)b * a.L + l_first) * a.C + n0 + cg;
+#pragma unroll 1
+            for (int r0 = lane / kLpr; r0 < ROWS; r0 += kBatch * kRpi) {
+                float4 acc[kBatch], gin[kBatch];
+                uint2 in[kBatch];
+                bool live[kBatch];
+#pragma unroll
+                for (int i = 0; i < kBatch; ++i) {
+                    const int r = r0 + kRpi * i, l = l_first + r;
+                    live[i] = l < a.L;
+                    acc[i] = *reinterpret_cast<const float4 *>(st + r * kStagePitch + cg);
+                    if (live[i]) {
+                        const int64_t o = row0 + (int64_t)(r * a.C);
+                        if constexpr (EPI == kEpiForward) {
+                            in[i] = *reinterpret_cast<const uint2 *>(a.x + o);
+                        } else {
+                            gin[i] = *reinterpret_cast<const float4 *>(a.gx + o);
+                            if (a.gzprev) in[i] = *reinterpret_cast<const uint2 *>(a.zprev + o);
+                        }
                     }
-                } else {
-                    float4 g = gin[i];
-                    g.x += acc[i].x, g.y += acc[i].y, g.z += acc[i].z, g.w += acc[i].w;
-                    *reinterpret_cast<float4 *>(a.gx + o) = g;
-                    if (a.gzprev) {
-                        const float2 z01 =
+                }
+#pragma unroll
+                for (int i = 0; i < kBatch; ++i) {
+                    if (!live[i]) continue;
+                    const int64_t o = row0 + (int64_t)((r0 + kRpi * i) * a.C);
+                    if constexpr (EPI == kEpiForward) {
+                        const float2 x01 =
                             __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&in[i].x));
-                        const float2 z23 =
+                        const float2 x23 =
                             __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&in[i].y));
-                        uint2 gv;
-                        *reinterpret_cast<__nv_bfloat162 *>(&gv.x) =
-                            __floats2bfloat162_rn(g.x * gelu_grad(z01.x), g.y * gelu_grad(z01.y));
-                        *reinterpret_cast<__nv_bfloat162 *>(&gv.y) =
-                            __floats2bfloat162_rn(g.z * gelu_grad(z23.x), g.w * gelu_grad(z23.y));
-                        *reinterpret_cast<uint2 *>(a.gzprev + o) = gv;
+                        const float z0 = acc[i].x + bias.x, z1 = acc[i].y + bias.y,
+                                    z2 = acc[i].z + bias.z, z3 = acc[i].w + bias.w;
+                        uint2 yv;
+                        *reinterpret_cast<__nv_bfloat162 *>(&yv.x) =
+                            __floats2bfloat162_rn(x01.x + gelu(z0), x01.y + gelu(z1));
+                        *reinterpret_cast<__nv_bfloat162 *>(&yv.y) =
+                            __floats2bfloat162_rn(x23.x + gelu(z2), x23.y + gelu(z3));
+                        *reinterpret_cast<uint2 *>(a.y + o) = yv;
+                        if (a.z) {
+                            uint2 zv;
+                            *reinterpret_cast<__nv_bfloat162 *>(&zv.x) = __floats2bfloat162_rn(z0, z1);
+                            *reinterpret_cast<__nv_bfloat162 *>(&zv.y) = __floats2bfloat162_rn(z2, z3);
+                            *reinterpret_cast<uint2 *>(a.z + o) = zv;
+                        }
+                    } else {
+                        float4 g = gin[i];
+                        g.x += acc[i].x, g.y += acc[i].y, g.z += acc[i].z, g.w += acc[i].w;
+                        *reinterpret_cast<float4 *>(a.gx + o) = g;
+                        if (a.gzprev) {
+                            const float2 z01 =
+                                __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&in[i].x));
+                            const float2 z23 =
+                                __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&in[i].y));
+                            uint2 gv;
+                            *reinterpret_cast<__nv_bfloat162 *>(&gv.x) =
+                                __floats2bfloat162_rn(g.x * gelu_grad(z01.x), g.y * gelu_grad(z01.y));
+                            *reinterpret_cast<__nv_bfloat162 *>(&gv.y) =
+                                __floats2bfloat162_rn(g.z * gelu_grad(z23.x), g.w * gelu_grad(z23.y));
+                            *reinterpret_cast<uint2 *>(a.gzprev + o) = gv;
+                        }
                     }
                 }
             }
         }
     }
     __syncwarp();  // the staging block is rewritten by the next tile
+}
+
+// The 128 x 128 form's epilogue of one warp, 32 rows x 32 columns: the
+// accumulator rows (one per lane after tcgen05.ld) go through a padded
+// shared-memory block so that global memory sees whole row segments.
+template <int EPI>
+__device__ __forceinline__ void epilogue_rows(const ConvArgs &a, float *st, uint32_t taddr, int b,
+                                              int l_first, int n0, bool skip)
+{
+    const int lane = threadIdx.x & 31;
+    float v[32];
+    __syncwarp();
+    tmem_ld32(taddr, v);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<float4 *>(st + lane * kStagePitch + 4 * j) =
+            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    __syncwarp();
+    finish_rows<EPI, 32>(a, st, b, l_first, n0, skip);
 }
 
 template <int EPI>
@@ -707,7 +796,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             __syncwarp();
             if (!ready) failed = 1;
             tc_fence_after();
-            epilogue_rows<EPI, 32>(a, staging + e * 32 * kStagePitch,
+            epilogue_rows<EPI>(a, staging + e * 32 * kStagePitch,
                                    tmem + acc * kTile + ((uint32_t)(quarter * 32) << 16) + col0, b,
                                    l0 + quarter * 32, n0 + col0, failed != 0);
             tc_fence_before();
@@ -921,7 +1010,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
                 for (int j = 0; j < kNStageRows; ++j) st[j * kStagePitch + lane] = v[j];
                 __syncwarp();
-                finish_rows<EPI, 32, kNStageRows>(a, st, b, l0 + pos0 + h, co0 + quarter * 32, failed != 0);
+                finish_rows<EPI, kNStageRows>(a, st, b, l0 + pos0 + h, co0 + quarter * 32, failed != 0);
             }
             tc_fence_before();
             __syncwarp();
@@ -1224,25 +1313,6 @@ __global__ void k_lift(const float *feat, const float *Wl, const float *bl, __nv
         }
         *reinterpret_cast<__nv_bfloat162 *>(x0 + p * C + c) = __floats2bfloat162_rn(acc0, acc1);
     }
-}
-
-// Two floats in a register pair and one fused multiply-add on both: the same
-// rounding as two scalar ones in half the issue slots.
-__device__ __forceinline__ uint64_t pack2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)

@@ -89,6 +89,24 @@ def test_bias_gradient(lib, P, C, skip):
     close(gb, before + gz.double().sum(0), before.abs() + gz.double().abs().sum(0))
 
 
+@pytest.mark.parametrize("impl", [0, 3])
+@pytest.mark.parametrize("B,L,C,k,d", [(1, 1, 128, 5, 4), (3, 300, 128, 5, 3), (2, 77, 256, 3, 2), (2, 257, 128, 5, 1),
+                                       (1200, 300, 128, 3, 1)])
+def test_forward_without_the_pre_activation(lib, impl, B, L, C, k, d):
+    """The inference product takes other accesses and packed arithmetic: the
+    same bits as the product that also stores the pre-activation."""
+    import torch
+    x, W, b = make(1, B * L, C, dtype="bfloat16"), make(2, k, C, C, dtype="bfloat16"), make(3, C)
+    y = [torch.full((B * L + 1, C), 7.0, device="cuda", dtype=torch.bfloat16) for _ in range(2)]
+    z = torch.empty(B * L, C, device="cuda", dtype=torch.bfloat16)
+    st = torch.zeros(1, device="cuda", dtype=torch.int32)
+    for out, pre in ((y[0], z.data_ptr()), (y[1], None)):
+        assert lib.lbm_nn_conv_forward(x.data_ptr(), W.data_ptr(), b.data_ptr(), out.data_ptr(), pre, B, L, C, k, d, impl,
+                                       st.data_ptr(), None) == 0
+    assert int(st) == 0 and torch.equal(y[0], y[1])
+    assert bool((y[0][B * L] == 7.0).all())
+
+
 @pytest.mark.parametrize("impl", [0, 1, 2, 3])
 @pytest.mark.parametrize("B,L,C,k,d", [(3, 300, 128, 5, 3), (1, 64, 128, 3, 1), (2, 77, 256, 3, 2), (40, 130, 128, 5, 1)])
 def test_bias_gradient_with_the_weight_gradient(lib, impl, B, L, C, k, d):
