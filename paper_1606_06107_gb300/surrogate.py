@@ -520,12 +520,11 @@ def fallback_windows(L: int, width: int, margin: int):
 
 
 def _latency_block(length: int) -> int:
-    """Block size of an ensemble run whose time is one problem's latency (a
-    few problems, or one wave of short ones): one node per thread, up to
-    1024.  The ensemble kernel steps a problem with one block, so a 4096-node
-    tube at 256 threads makes each thread update 16 nodes in turn per step
-    (32 steps: 1.02 ms, against 0.45 ms at 1024 threads; 1024 windows of 384
-    nodes: 0.368 ms at 256 threads, 0.355 ms at 384)."""
+    """Nodes a block updates at a time (two per thread) in an ensemble run
+    whose time is one problem's latency (a few problems, or one wave of short
+    ones): the whole problem, up to 1024.  The ensemble kernel steps a problem
+    with one block, so fewer would make each thread update several pairs in
+    turn per step."""
     return int(min(1024, max(32, -(-length // 32) * 32)))
 
 
