@@ -499,14 +499,19 @@ int lbm_step(lbm_handle h, int64_t k)
     DeviceGuard g(h->device);
     Args a = make_args(h);
     if (h->lattice == LBM_D1Q7 && lbm::tube_steps_ok(a, k)) {
-        const int end = h->cur ^ (int)(k & 1);  // the buffer single steps would end in
-        a.src = h->buf[h->cur];
-        a.dst = h->buf[end];
-        ++h->launches;
-        const cudaError_t e = lbm::launch_tube_steps(a, k, h->stream);
-        if (e != cudaSuccess) return cuda_fail(h, e, "tube kernel");
-        h->cur = end;
-        h->steps += k;
+        // (a launch of 2^16 steps runs for some 0.05-0.2 s)
+        for (int64_t left = k; left > 0;) {
+            const int64_t run = std::min<int64_t>(left, 1 << 16);
+            const int end = h->cur ^ (int)(run & 1);  // the buffer single steps would end in
+            a.src = h->buf[h->cur];
+            a.dst = h->buf[end];
+            ++h->launches;
+            const cudaError_t e = lbm::launch_tube_steps(a, run, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "tube kernel");
+            h->cur = end;
+            h->steps += run;
+            left -= run;
+        }
         return LBM_OK;
     }
     for (int64_t s = 0; s < k; ++s) {
