@@ -17,6 +17,7 @@
 // lbm_step_node.cuh); every kernel is instantiated per storage type.  One
 // thread owns one node; a block is 128 consecutive x positions of one row.
 #pragma once
+#include <atomic>
 #include <cstdint>
 #include <type_traits>
 #include <cuda_bf16.h>
@@ -51,7 +52,16 @@ template <typename ST, int MODE> struct StepMinBlocks {
     static constexpr int value = (std::is_same<ST, float>::value || MODE != 0) ? 4 : 5;
 #endif
 };
-#define LBM_STEP_BOUNDS __launch_bounds__(kBlockX, StepMinBlocks<ST, MODE>::value)
+// Float FD steps of more than one wave at four blocks per SM take the kernel
+// compiled for three (168 registers): they are bound by the latency of 4-7
+// loads per population from L2, and more of them in flight are worth more than
+// more warps.  600 x 420 D2Q37 38.1 -> 30.6 us, 2048 x 1024 D2Q49 367 -> 285; a
+// single wave loses (300 x 200 D2Q49, n = 0, 600 blocks: 10.3 -> 11.4), and five
+// or six blocks spill (50.5 / 53.7 us at 600 x 420).
+#ifndef LBM_FD_WIDE_BLOCKS
+#define LBM_FD_WIDE_BLOCKS 3
+#endif
+constexpr int kFdWideBlocks = LBM_FD_WIDE_BLOCKS;
 
 // ---------------------------------------------------------------------------
 // Velocity sets.  xi_i = r * e_i; order (ez, ey, ex) ascending.  The sets are
@@ -791,8 +801,8 @@ __device__ __forceinline__ void collide_store(const Params<Lattice<LAT>::Q, ST> 
 // cp.async.bulk + an mbarrier ran 27 % slower -- blocks idle while their
 // copies land and the smem per block halves the resident warps -- and
 // cp.async.bulk.prefetch.L2 of rows 16..128 ahead ran 4..27 % slower.)
-template <int LAT, bool ROT, int MODE, typename ST>
-__global__ void LBM_STEP_BOUNDS k_step(const Params<Lattice<LAT>::Q, ST> p)
+template <int LAT, bool ROT, int MODE, typename ST, int MINB = StepMinBlocks<ST, MODE>::value>
+__global__ void __launch_bounds__(kBlockX, MINB) k_step(const Params<Lattice<LAT>::Q, ST> p)
 {
     using L = Lattice<LAT>;
     constexpr int Q = L::Q;
@@ -1133,6 +1143,21 @@ __global__ void __launch_bounds__(kBlockX) k_set_state(const Params<Lattice<LAT>
 // ---------------------------------------------------------------------------
 // Host-side dispatch for one lattice.
 
+// SMs of the current device, looked up once per device (a launch that is being
+// captured queries nothing); 152 where the lookup fails.
+inline int device_sms()
+{
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    int n = known[dev].load();
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 152;
+        known[dev].store(n);
+    }
+    return n;
+}
+
 // Launch that may start while the kernel before it on the stream is still
 // running (programmatic dependent launch): `kernel` calls pdl_wait() before
 // its first global access, so only its launch and its index arithmetic
@@ -1183,6 +1208,10 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
             // per-node references: the deviation-space kernel (STREAM only)
             return launch_pdl(k_step_node<LAT, ROT, ST>, grid, block, 0, s, p);
         } else {
+            if constexpr (MODE == 1 && std::is_same<ST, float>::value && Lattice<LAT>::D == 2) {
+                if ((int64_t)grid.x * grid.y > 4 * (int64_t)device_sms())
+                    return launch_pdl(k_step<LAT, ROT, MODE, ST, kFdWideBlocks>, grid, block, 0, s, p);
+            }
             return launch_pdl(k_step<LAT, ROT, MODE, ST>, grid, block, 0, s, p);
         }
         break;
