@@ -194,12 +194,9 @@ template <typename N> struct NodeStorage {
 };
 template <> struct Storage<NodeHalf> : NodeStorage<NodeHalf> {};
 template <> struct Storage<NodeBf16> : NodeStorage<NodeBf16> {};
-using ::__ldcg;  // keep CUDA's overloads visible beside the two below
-using ::__ldg;
+using ::__ldg;  // keep CUDA's overloads visible beside the two below
 __device__ __forceinline__ NodeHalf __ldg(const NodeHalf *a) { return NodeHalf{::__ldg(&a->v)}; }
 __device__ __forceinline__ NodeBf16 __ldg(const NodeBf16 *a) { return NodeBf16{::__ldg(&a->v)}; }
-__device__ __forceinline__ NodeHalf __ldcg(const NodeHalf *a) { return NodeHalf{::__ldcg(&a->v)}; }
-__device__ __forceinline__ NodeBf16 __ldcg(const NodeBf16 *a) { return NodeBf16{::__ldcg(&a->v)}; }
 
 // ---------------------------------------------------------------------------
 // Kernel parameters (passed by value: they live in the constant bank, so the
@@ -381,20 +378,14 @@ __device__ __forceinline__ Offsets node_offsets(const Params<Q, ST> &p, int x, i
     return o;
 }
 
-// CG = 0: read-only path (the source buffer is never written during the
-// launch).  CG = 1: L2-coherent loads, for kernels that read back what the
-// same launch wrote (the persistent ensemble kernel).  CG = 2: plain
-// generic loads (a state held in shared memory).
-template <int CG = 0, int Q, typename ST>
+// Read-only path: the source buffer is never written during the launch.
+template <int Q, typename ST>
 __device__ __forceinline__ float ld(const Params<Q, ST> &p, int pop, int off)
 {
     // 32-bit element index up to 49 populations; D3Q343 states exceed 2^32
     using Idx = typename std::conditional<(Q > 49), uint64_t, uint32_t>::type;
     const ST *a = p.src + ((Idx)pop * (Idx)p.S + (Idx)(uint32_t)off);
-    ST v;
-    if constexpr (CG == 2) v = *a;
-    else if constexpr (CG == 1) v = __ldcg(a);
-    else v = __ldg(a);
+    const ST v = __ldg(a);
     if constexpr (std::is_same<ST, float>::value) return v;
     else {
         const float w = pop < Q ? p.w[pop] : p.wr[pop - Q];
@@ -621,7 +612,7 @@ __device__ __forceinline__ void heq_node(const Params<Q, ST> &p, float T, float 
 // convection by u at Courant number u * nu_scale, BGK toward h^eq(T).
 // (Issuing these neighbour loads right after the moments, before the
 // translational work, measured 9 % slower on the 2048^2 workload.)
-template <int D, int CG = 0, int Q, typename ST>
+template <int D, int Q, typename ST>
 __device__ __forceinline__ void rot_advect(const Params<Q, ST> &p, const Offsets &o,
                                            const float *h, const Moments &m, float *adv)
 {
@@ -639,8 +630,8 @@ __device__ __forceinline__ void rot_advect(const Params<Q, ST> &p, const Offsets
         const float anu = fabsf(nu[a]);
 #pragma unroll
         for (int j = 0; j < 7; ++j)
-            adv[j] += upwind_abs(anu, ld<CG>(p, Q + j, uu), ld<CG>(p, Q + j, u1), h[j],
-                                 ld<CG>(p, Q + j, d1));
+            adv[j] += upwind_abs(anu, ld(p, Q + j, uu), ld(p, Q + j, u1), h[j],
+                                 ld(p, Q + j, d1));
     }
 }
 
@@ -659,7 +650,7 @@ __device__ __forceinline__ void rot_store(const Params<Q, ST> &p, int self, cons
 // Load the time-t populations of one node.  STREAM: pull g_i(x) = ft_i(x - e_i).
 // FD: g_i(x) = ft_i(x).
 
-template <int LAT, bool ROT, int MODE, int CG = 0, int Q, typename ST>
+template <int LAT, bool ROT, int MODE, int Q, typename ST>
 __device__ __forceinline__ void load_node(const Params<Q, ST> &p, const Offsets &o, float *g,
                                           float *h)
 {
@@ -669,18 +660,18 @@ __device__ __forceinline__ void load_node(const Params<Q, ST> &p, const Offsets 
         const int off = (MODE == 0)
                             ? o.z[3 - L::ez(i)] + o.y[3 - L::ey(i)] + o.x[3 - L::ex(i)]
                             : o.self();
-        g[i] = ld<CG>(p, i, off);
+        g[i] = ld(p, i, off);
     }
     if (ROT) {
 #pragma unroll
-        for (int j = 0; j < 7; ++j) h[j] = ld<CG>(p, L::Q + j, o.self());
+        for (int j = 0; j < 7; ++j) h[j] = ld(p, L::Q + j, o.self());
     }
 }
 
 // FD transport of one translational population (Eq. DisEvolSpaTiI): the
 // upwind side of each axis is fixed by the sign of e_ia, the Courant number
 // is |e_ia| / m.
-template <int LAT, int I, int CG = 0, int Q, typename ST>
+template <int LAT, int I, int Q, typename ST>
 __device__ __forceinline__ float fd_convect(const Params<Q, ST> &p, const Offsets &o, float g0)
 {
     using L = Lattice<LAT>;
@@ -693,17 +684,17 @@ __device__ __forceinline__ float fd_convect(const Params<Q, ST> &p, const Offset
         const int rest = o.self() - oa[3];
         const bool pos = e[a] > 0;
         const float anu = (float)(pos ? e[a] : -e[a]) * p.inv_m;
-        adv += upwind_abs(anu, ld<CG>(p, I, rest + (pos ? oa[1] : oa[5])),
-                          ld<CG>(p, I, rest + (pos ? oa[2] : oa[4])), g0,
-                          ld<CG>(p, I, rest + (pos ? oa[4] : oa[2])));
+        adv += upwind_abs(anu, ld(p, I, rest + (pos ? oa[1] : oa[5])),
+                          ld(p, I, rest + (pos ? oa[2] : oa[4])), g0,
+                          ld(p, I, rest + (pos ? oa[4] : oa[2])));
     }
     return adv;
 }
 
-template <int LAT, int MODE, int I, int CG = 0, int Q, typename ST>
+template <int LAT, int MODE, int I, int Q, typename ST>
 __device__ __forceinline__ float transport(const Params<Q, ST> &p, const Offsets &o, float g0)
 {
-    if constexpr (MODE == 1) return fd_convect<LAT, I, CG>(p, o, g0);
+    if constexpr (MODE == 1) return fd_convect<LAT, I>(p, o, g0);
     return 0.f;
 }
 
@@ -1006,13 +997,13 @@ __global__ void __launch_bounds__(kBlockX) k_init(const Params<Lattice<LAT>::Q, 
 // ---------------------------------------------------------------------------
 // rho, u, T of the current state into unpadded caller arrays.
 
-template <int LAT, bool ROT, int MODE, int CG = 0, typename ST>
+template <int LAT, bool ROT, int MODE, typename ST>
 __device__ __forceinline__ void moments_node(const Params<Lattice<LAT>::Q, ST> &p, int x, int y, int z)
 {
     using L = Lattice<LAT>;
     const Offsets o = node_offsets<L::D>(p, x, y, z);
     float g[L::Q], h[7];
-    load_node<LAT, ROT, MODE, CG>(p, o, g, h);
+    load_node<LAT, ROT, MODE>(p, o, g, h);
     const Moments m = node_moments<LAT, ROT>(p, g, h);
     const int64_t node = ((int64_t)z * p.Y + y) * p.X + x;
     p.out0[node] = m.rho;
@@ -1204,6 +1195,8 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
     case Op::Step:
         if constexpr (LAT == 4) {  // 343 populations: the two-pass kernel
             return launch_step_q343<ROT, ST>(a, s);
+        } else if constexpr (LAT == 1 && std::is_same<ST, float>::value) {
+            return cudaErrorInvalidValue;  // lbm_d1q7.cu has its own
         } else if constexpr (NodeRef<ST>::value) {
             // per-node references: the deviation-space kernel (STREAM only)
             return launch_pdl(k_step_node<LAT, ROT, ST>, grid, block, 0, s, p);
