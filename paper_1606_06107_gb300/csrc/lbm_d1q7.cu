@@ -45,17 +45,19 @@ template <bool ROT, int MODE> __global__ void __launch_bounds__(kBlockX) k_tube_
     for (int k = 0; k < 7; ++k) o[k] = bc_wrap(x + k - 3, p.X, p.bc);
     pdl_wait();
     pdl_trigger();
-    float rho, T;
+    float out[ROT ? 14 : 7], rho, T;  // stored together: no load waits for a store
     tube_update<ROT, MODE, float>(
-        p.lat, p.rates, [&](int pop, int d) { return __ldg(p.src + (uint32_t)pop * (uint32_t)p.S + o[3 + d]); },
+        p.lat, p.rates, [&](int pop, int d) { return __ldca(p.src + ((uint32_t)pop * (uint32_t)p.S + (uint32_t)o[3 + d])); },
         [&](float ux) {
             const bool pos = ux >= 0.f;
             const int u2 = pos ? o[1] : o[5], u1 = pos ? o[2] : o[4], d1 = pos ? o[4] : o[2];
             return [&p, u2, u1, d1](int j, int k) {
-                return __ldg(p.src + (uint32_t)(7 + j) * (uint32_t)p.S + (k == 2 ? u2 : k == 1 ? u1 : d1));
+                return __ldca(p.src + ((uint32_t)(7 + j) * (uint32_t)p.S + (uint32_t)(k == 2 ? u2 : k == 1 ? u1 : d1)));
             };
         },
-        [&](int pop, float v) { p.dst[(uint32_t)pop * (uint32_t)p.S + x] = v; }, rho, T);
+        [&](int pop, float v) { out[pop] = v; }, rho, T);
+#pragma unroll
+    for (int i = 0; i < (ROT ? 14 : 7); ++i) p.dst[(uint32_t)i * (uint32_t)p.S + (uint32_t)x] = out[i];
     if (tube_bad(rho, T)) atomicOr(p.status, 1);
 }
 

@@ -37,7 +37,7 @@ constexpr int kQ343Block = 128;
 // index: the state of a 384^3 grid holds 2 x 10^10 values).
 __device__ __forceinline__ float q343_load(const Params<kQ343> &p, int i, int off)
 {
-    return __ldg(p.src + ((uint64_t)i * (uint64_t)p.S + (uint64_t)(uint32_t)off));
+    return ld_ro(p.src + ((uint64_t)i * (uint64_t)p.S + (uint64_t)(uint32_t)off));
 }
 __device__ __forceinline__ void q343_store(const Params<kQ343> &p, int i, int self, float v)
 {
@@ -521,8 +521,6 @@ __global__ void __launch_bounds__(kPairBlock, LBM_Q343_PAIR_MIN_BLOCKS)
     const PairOffsets o = pair_offsets(p, x, y);
     extern __shared__ unsigned char q343_smem[];
     uint32_t *stash = reinterpret_cast<uint32_t *>(q343_smem);
-    pdl_wait();
-    pdl_trigger();
     const Q343PairSums s = q343_pair_sums<kPairStash, WHOLE>(p, o, z, stash);
     q343_pair_collide<ROT, kPairStash, WHOLE>(p, qw, o, x, z, s, stash);
 }
@@ -550,7 +548,13 @@ __global__ void __launch_bounds__(kQ343Block, 4) k_moments_q343_pair(const Param
     }
 }
 
-// Float storage, one launch: pass 1, then pass 2 on the same thread.
+// Float storage, one launch: pass 1, then pass 2 on the same thread.  The two
+// step kernels are not launched dependently: pass 2 interleaves its loads with
+// its stores and needs the read-only path (see ld), which a kernel that is
+// resident while its predecessor writes may not use.  With ordinary loads and
+// the dependent launch, the next row loaded ahead: 101 x 96 x 90 float n = 4
+// 0.83-0.89 ms a step against 0.775; 256^3 half n = 0 / n = 4 8.15 / 9.13
+// against 7.70 / 8.63.
 template <bool ROT>
 __global__ void __launch_bounds__(kQ343Block, LBM_Q343_MIN_BLOCKS)
     k_step_q343(const Params<kQ343> p, const Q343Weights qw)
@@ -559,8 +563,6 @@ __global__ void __launch_bounds__(kQ343Block, LBM_Q343_MIN_BLOCKS)
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.X) return;
     const Offsets o = node_offsets<3>(p, x, y, z);
-    pdl_wait();
-    pdl_trigger();
     q343_collide<ROT>(p, qw, o, z, q343_sums(p, o, z));
 }
 
@@ -644,14 +646,16 @@ template <bool ROT, typename ST> cudaError_t launch_step_q343(const Args &a, cud
     qw.iw_unit = (float)(1.0 / ((double)a.wr[2] * (double)a.wr[3] * (double)a.wr[3]));
     if constexpr (std::is_same<ST, float>::value) {
         const dim3 grid((a.X + kQ343Block - 1) / kQ343Block, a.Y, a.Z);
-        return launch_pdl(k_step_q343<ROT>, grid, dim3(kQ343Block), 0, s, p, qw);
+        k_step_q343<ROT><<<grid, kQ343Block, 0, s>>>(p, qw);
+        return cudaGetLastError();
     } else {
         const dim3 grid((a.X + 2 * kPairBlock - 1) / (2 * kPairBlock), a.Y, a.Z);
         auto go = [&](auto whole) {
             constexpr bool W = decltype(whole)::value;
             const cudaError_t e = allow_smem<k_step_q343_pair<ROT, W, ST>>(kPairStashBytes);
             if (e != cudaSuccess) return e;
-            return launch_pdl(k_step_q343_pair<ROT, W, ST>, grid, dim3(kPairBlock), kPairStashBytes, s, p, qw);
+            k_step_q343_pair<ROT, W, ST><<<grid, kPairBlock, kPairStashBytes, s>>>(p, qw);
+            return cudaGetLastError();
         };
         return pair_whole(a) ? go(std::true_type{}) : go(std::false_type{});
     }

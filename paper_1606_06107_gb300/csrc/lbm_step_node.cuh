@@ -82,15 +82,15 @@ k_step_node(const Params<Lattice<LAT>::Q, ST> p)
         constexpr int I = decltype(ic)::value;
         constexpr int ex = L::ex(I), ey = L::ey(I);
         const int off = oy[3 - ey] + ox[3 - ex];
-        d[I] = DV::get(__ldg(src + ((uint32_t)I * S + (uint32_t)off)));
-        d[I] += ref_dev(p, I, __ldg(p.ref_src + off), (float)ex, (float)ey, p.kmD[I], p.kt2[I]);
+        d[I] = DV::get(src[(uint32_t)I * S + (uint32_t)off]);
+        d[I] += ref_dev(p, I, p.ref_src[off], (float)ex, (float)ey, p.kmD[I], p.kt2[I]);
     });
     float t_self = 0.f;
     if (ROT) {
-        t_self = ref_t(__ldg(p.ref_src + self));
+        t_self = ref_t(p.ref_src[self]);
 #pragma unroll
         for (int j = 0; j < 7; ++j) {
-            h[j] = DV::get(__ldg(src + ((uint32_t)(Q + j) * S + (uint32_t)self)));
+            h[j] = DV::get(src[(uint32_t)(Q + j) * S + (uint32_t)self]);
             h[j] += t_self * fmaf(t_self, p.hb[j], p.ha[j]);
         }
     }
@@ -206,12 +206,12 @@ k_step_node(const Params<Lattice<LAT>::Q, ST> p)
 #pragma unroll
             for (int j = 0; j < 7; ++j) {
                 const uint32_t o = (uint32_t)(Q + j) * S;
-                adv[j] += upwind_abs(anu, DV::get(__ldg(src + (o + (uint32_t)uu))),
-                                     DV::get(__ldg(src + (o + (uint32_t)u1))), h[j],
-                                     DV::get(__ldg(src + (o + (uint32_t)d1))));
+                adv[j] += upwind_abs(anu, DV::get(src[o + (uint32_t)uu]),
+                                     DV::get(src[o + (uint32_t)u1]), h[j],
+                                     DV::get(src[o + (uint32_t)d1]));
             }
-            const float tuu = ref_t(__ldg(p.ref_src + uu)), tu1 = ref_t(__ldg(p.ref_src + u1));
-            const float td1 = ref_t(__ldg(p.ref_src + d1));
+            const float tuu = ref_t(p.ref_src[uu]), tu1 = ref_t(p.ref_src[u1]);
+            const float td1 = ref_t(p.ref_src[d1]);
             adv_t1 += upwind_abs(anu, tuu, tu1, 0.f, td1);
             adv_t2 += upwind_abs(anu, tuu * tuu, tu1 * tu1, 0.f, td1 * td1);
         };

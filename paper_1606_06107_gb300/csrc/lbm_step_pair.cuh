@@ -122,9 +122,9 @@ __device__ __forceinline__ uint32_t ld_pair(const Params<Q, ST> &p, int pop, int
     const unsigned short *src = reinterpret_cast<const unsigned short *>(p.src);
     const Idx at = (Idx)pop * (Idx)p.S + (Idx)(uint32_t)row;
     if (WHOLE && (d & 1) == 0)
-        return __ldg(reinterpret_cast<const uint32_t *>(src + (at + (Idx)(uint32_t)o.x[d + 3])));
-    const uint32_t a = __ldg(src + (at + (Idx)(uint32_t)o.x[d + 3]));
-    const uint32_t b = __ldg(src + (at + (Idx)(uint32_t)o.x[d + 4]));
+        return ld_ro(reinterpret_cast<const uint32_t *>(src + (at + (Idx)(uint32_t)o.x[d + 3])));
+    const uint32_t a = ld_ro(src + (at + (Idx)(uint32_t)o.x[d + 3]));
+    const uint32_t b = ld_ro(src + (at + (Idx)(uint32_t)o.x[d + 4]));
     return __byte_perm(a, b, 0x5410);
 }
 

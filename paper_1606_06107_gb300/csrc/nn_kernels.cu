@@ -106,6 +106,10 @@ __device__ __forceinline__ uint4 pack8(const float *v)
 // before its first global access.  pdl_trigger() lets the next one start its
 // own set-up.  (A kernel launched without the attribute, such as the weights'
 // cast, never overlaps: what it wrote is there when any of these starts.)
+// These kernels read global memory with ordinary loads, never through the
+// read-only path (__ldg, const __restrict__): that one is defined for data
+// nobody writes during the kernel's lifetime, which begins while the
+// predecessor still writes, and its loads may be moved above the wait.
 // Loss and gradients of a 32 x 4096 minibatch 634 -> 580 us.
 __device__ __forceinline__ void pdl_chain()
 {
@@ -313,7 +317,7 @@ __device__ __forceinline__ void epilogue32(const ConvArgs &a, const float (&v)[3
             unpack8(*reinterpret_cast<const uint4 *>(a.x + base + c + 8 * q), xr);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const float zz = v[8 * q + j] + __ldg(a.bias + n0 + c + 8 * q + j);
+                const float zz = v[8 * q + j] + a.bias[n0 + c + 8 * q + j];
                 zv[j] = zz;
                 yv[j] = xr[j] + gelu(zz);
             }
@@ -573,7 +577,7 @@ __device__ __forceinline__ void finish_rows(const ConvArgs &a, const float *st, 
             uint64_t bias[4];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(a.bias + n0 + cg) + q);
+                const float4 v = reinterpret_cast<const float4 *>(a.bias + n0 + cg)[q];
                 bias[2 * q] = pack2(v.x, v.y);
                 bias[2 * q + 1] = pack2(v.z, v.w);
             }
@@ -1285,8 +1289,8 @@ __global__ void k_lift(const float *feat, const float *Wl, const float *bl, __nv
     float w0[F], w1[F];
 #pragma unroll
     for (int j = 0; j < F / 4; ++j) {
-        const float4 q0 = __ldg(reinterpret_cast<const float4 *>(Wl + c * F) + j);
-        const float4 q1 = __ldg(reinterpret_cast<const float4 *>(Wl + (c + 1) * F) + j);
+        const float4 q0 = reinterpret_cast<const float4 *>(Wl + c * F)[j];
+        const float4 q1 = reinterpret_cast<const float4 *>(Wl + (c + 1) * F)[j];
         w0[4 * j] = q0.x, w0[4 * j + 1] = q0.y, w0[4 * j + 2] = q0.z, w0[4 * j + 3] = q0.w;
         w1[4 * j] = q1.x, w1[4 * j + 1] = q1.y, w1[4 * j + 2] = q1.z, w1[4 * j + 3] = q1.w;
     }
@@ -1294,7 +1298,7 @@ __global__ void k_lift(const float *feat, const float *Wl, const float *bl, __nv
     const int64_t p0 = blockIdx.x * per_block, p1 = std::min(P, p0 + per_block);
     const int n4 = (int)(p1 - p0) * (F / 4);
     const float4 *src = reinterpret_cast<const float4 *>(feat + p0 * F);
-    for (int e = threadIdx.x; e < n4; e += blockDim.x) fsh[e] = __ldg(src + e);
+    for (int e = threadIdx.x; e < n4; e += blockDim.x) fsh[e] = src[e];
     __syncthreads();
     for (int64_t p = p0 + par; p < p1; p += 2) {
         const float4 *f = fsh + (p - p0) * (F / 4);
@@ -1362,7 +1366,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
     for (int q = 0; q < NP; ++q)
 #pragma unroll
-        for (int o = 0; o < FP; o += 2) acc[q][o / 2] = pack2(__ldg(bp + o), o + 1 < FO ? __ldg(bp + o + 1) : 0.f);
+        for (int o = 0; o < FP; o += 2) acc[q][o / 2] = pack2(bp[o], o + 1 < FO ? bp[o + 1] : 0.f);
     for (int k = 0; k < chunks; ++k) {
         if (k + 1 < chunks) {
             fetch(k + 1);
@@ -1446,7 +1450,7 @@ __global__ void __launch_bounds__(256) k_head_bwd(const float *gout, const __nv_
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             accW[o][j] = 0.f;
-            if constexpr (WREG) w[o][j] = __ldg(Wp + o * C + chan(j));
+            if constexpr (WREG) w[o][j] = Wp[o * C + chan(j)];
         }
     }
     // the next position's values are in flight while one is worked on
@@ -1457,13 +1461,13 @@ __global__ void __launch_bounds__(256) k_head_bwd(const float *gout, const __nv_
     } next;
     auto fetch = [&](int64_t p) {
 #pragma unroll
-        for (int o = 0; o < FO; ++o) next.go[o] = __ldg(gout + p * FO + o);
+        for (int o = 0; o < FO; ++o) next.go[o] = gout[p * FO + o];
         if constexpr (VEC) {
 #pragma unroll
             for (int v = 0; v < NJ / 4; ++v) {
                 const int64_t c = p * C + 4 * lane + 128 * v;
-                next.xq[v] = __ldg(reinterpret_cast<const uint2 *>(x + c));
-                next.zq[v] = __ldg(reinterpret_cast<const uint2 *>(z + c));
+                next.xq[v] = *reinterpret_cast<const uint2 *>(x + c);
+                next.zq[v] = *reinterpret_cast<const uint2 *>(z + c);
             }
         } else {
 #pragma unroll
@@ -1505,7 +1509,7 @@ __global__ void __launch_bounds__(256) k_head_bwd(const float *gout, const __nv_
             g[j] = 0.f;
 #pragma unroll
             for (int o = 0; o < FO; ++o) {
-                g[j] = fmaf(go[o], WREG ? w[WREG ? o : 0][j] : __ldg(Wp + o * C + chan(j)), g[j]);
+                g[j] = fmaf(go[o], WREG ? w[WREG ? o : 0][j] : Wp[o * C + chan(j)], g[j]);
                 accW[o][j] = fmaf(go[o], xv[j], accW[o][j]);
             }
         }
@@ -1565,14 +1569,14 @@ __global__ void __launch_bounds__(1024) k_lift_bwd(const float *gx0, const float
     const int c = threadIdx.x % C, r = threadIdx.x / C, R = blockDim.x / C;
     const int64_t p0 = (int64_t)blockIdx.x * per_block;
     const int n = (int)std::min<int64_t>(per_block, P - p0);
-    for (int e = threadIdx.x; e < n * F; e += blockDim.x) sh[e] = __ldg(feat + p0 * F + e);
+    for (int e = threadIdx.x; e < n * F; e += blockDim.x) sh[e] = feat[p0 * F + e];
     __syncthreads();
     float acc[F], accb = 0.f;
 #pragma unroll
     for (int j = 0; j < F; ++j) acc[j] = 0.f;
 #pragma unroll 8
     for (int q = r; q < n; q += R) {
-        const float g = __ldg(gx0 + (p0 + q) * C + c);
+        const float g = gx0[(p0 + q) * C + c];
         accb += g;
 #pragma unroll
         for (int j = 0; j < F / 4; ++j) {
@@ -1625,7 +1629,7 @@ __global__ void __launch_bounds__(256) k_colsum8(const __nv_bfloat16 *gz, float 
 #pragma unroll 8
     for (int64_t p = p0 + ty; p < p1; p += 16) {
         float v[8];
-        unpack8(__ldg(reinterpret_cast<const uint4 *>(base + p * C)), v);
+        unpack8(*reinterpret_cast<const uint4 *>(base + p * C), v);
 #pragma unroll
         for (int j = 0; j < 8; ++j) s[j] += v[j];
     }
@@ -1729,13 +1733,20 @@ __global__ void k_mse(const float *out, const float *target, float *gout, double
 {
     pdl_chain();
     double acc = 0.0;
-#pragma unroll 4
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float d = __ldg(out + i) - __ldg(target + i);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    auto put = [&](int64_t at, float d) {
         acc += (double)d * d;
-        if (gout) gout[i] = 2.0f * d / (float)n;
+        if (gout) gout[at] = 2.0f * d / (float)n;
+    };
+    for (; i + 3 * stride < n; i += 4 * stride) {  // four loads in flight before the first store
+        float d[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = out[i + k * stride] - target[i + k * stride];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) put(i + k * stride, d[k]);
     }
+    for (; i < n; i += stride) put(i, out[i] - target[i]);
     __shared__ double red[32];
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -1757,7 +1768,7 @@ struct Scale3 { float s[3]; };
 // nodes: features 33.4 -> 24.0 us, update 28.9 -> 19.2; 2^17 nodes: features
 // 4.0 -> 5.0, targets 5.1 -> 5.9 (a quarter of the blocks): from kVecNodes on.
 constexpr int64_t kVecNodes = 1 << 20;
-__device__ __forceinline__ float4 ldg4(const float *p, int64_t i) { return __ldg(reinterpret_cast<const float4 *>(p) + i); }
+__device__ __forceinline__ float4 ld4(const float *p, int64_t i) { return reinterpret_cast<const float4 *>(p)[i]; }
 
 template <bool VEC>
 __global__ void k_features(const float *rho, const float *u, const float *T, const float *gamma,
@@ -1772,10 +1783,10 @@ __global__ void k_features(const float *rho, const float *u, const float *T, con
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
          i += (int64_t)gridDim.x * blockDim.x) {
         if constexpr (VEC) {
-            const float4 r = ldg4(rho, i), v = ldg4(u, i), t = ldg4(T, i);
+            const float4 r = ld4(rho, i), v = ld4(u, i), t = ld4(T, i);
             // (32-bit division where it serves)
             const int64_t b = n <= 0x7fffffff ? (int64_t)((uint32_t)(4 * i) / (uint32_t)L) : 4 * i / L;
-            const float g = __ldg(gamma + b);
+            const float g = gamma[b];
             put(4 * i, r.x, v.x, t.x, g);
             put(4 * i + 1, r.y, v.y, t.y, g);
             put(4 * i + 2, r.z, v.z, t.z, g);
@@ -1796,8 +1807,8 @@ __global__ void k_targets(const float *rho, const float *u, const float *T, cons
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
          i += (int64_t)gridDim.x * blockDim.x) {
         if constexpr (VEC) {
-            const float4 r = ldg4(rho, i), v = ldg4(u, i), t = ldg4(T, i);
-            const float4 r2 = ldg4(rho2, i), v2 = ldg4(u2, i), t2 = ldg4(T2, i);
+            const float4 r = ld4(rho, i), v = ld4(u, i), t = ld4(T, i);
+            const float4 r2 = ld4(rho2, i), v2 = ld4(u2, i), t2 = ld4(T2, i);
             auto q = [&](float x2, float x, int k) { return (x2 - x) / sc.s[k]; };
             float4 *o = reinterpret_cast<float4 *>(target) + 3 * i;
             o[0] = make_float4(q(r2.x, r.x, 0), q(v2.x, v.x, 1), q(t2.x, t.x, 2), q(r2.y, r.y, 0));
@@ -1821,8 +1832,8 @@ __global__ void k_apply(const float *rho, const float *u, const float *T, const 
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
          i += (int64_t)gridDim.x * blockDim.x) {
         if constexpr (VEC) {
-            const float4 r = ldg4(rho, i), v = ldg4(u, i), t = ldg4(T, i);
-            const float4 a = ldg4(out, 3 * i), b = ldg4(out, 3 * i + 1), c = ldg4(out, 3 * i + 2);
+            const float4 r = ld4(rho, i), v = ld4(u, i), t = ld4(T, i);
+            const float4 a = ld4(out, 3 * i), b = ld4(out, 3 * i + 1), c = ld4(out, 3 * i + 2);
             auto q = [&](float x, float d, int k) { return fmaf(d, sc.s[k], x); };
             reinterpret_cast<float4 *>(rho2)[i] = make_float4(q(r.x, a.x, 0), q(r.y, a.w, 0), q(r.z, b.z, 0), q(r.w, c.y, 0));
             reinterpret_cast<float4 *>(u2)[i] = make_float4(q(v.x, a.y, 1), q(v.y, b.x, 1), q(v.z, b.w, 1), q(v.w, c.z, 1));
