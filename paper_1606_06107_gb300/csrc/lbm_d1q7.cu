@@ -155,12 +155,8 @@ template <bool ROT, int MODE, int MAXT> cudaError_t launch_tube_t(const Args &a,
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cfg.dynamicSmemBytes > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_tube_steps<ROT, MODE, MAXT>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)cfg.dynamicSmemBytes);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem<k_tube_steps<ROT, MODE, MAXT>>(sizeof(float) * 2 * kNodePitch * (MAXT + 6));
+    if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, k_tube_steps<ROT, MODE, MAXT>, p, steps, nodes);
 }
 

@@ -14,8 +14,6 @@
 // with the float32 moment corrections, as in the one- and two-dimensional
 // kernels.  Element indices are 64-bit (the state of a 384^3 grid holds
 // 2 x 10^10 values).
-#include <atomic>
-
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -610,24 +608,6 @@ template <bool ROT, typename ST> cudaError_t launch_moments_q343(const Args &a, 
     k_moments_q343<ROT><<<grid, kQ343Block, 0, s>>>(p);
     return cudaGetLastError();
     }
-}
-
-// The opt-in limit of dynamic shared memory is a function attribute, set once
-// per device.
-template <auto KERNEL> cudaError_t allow_smem(size_t bytes)
-{
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    static std::atomic<bool> done[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!done[dev].load()) {
-        e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        done[dev].store(true);
-    }
-    return cudaSuccess;
 }
 
 template <bool ROT, typename ST> cudaError_t launch_step_q343(const Args &a, cudaStream_t s)

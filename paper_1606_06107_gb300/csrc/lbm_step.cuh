@@ -1176,6 +1176,25 @@ inline int device_sms()
     return n;
 }
 
+// The opt-in limit of dynamic shared memory is an attribute of the kernel on a
+// device, which all handles and host threads share: it is set once, to the most
+// that any launch of the kernel takes (`bytes`), and never lowered.
+template <auto KERNEL> cudaError_t allow_smem(size_t bytes)
+{
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    static std::atomic<bool> done[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!done[dev].load()) {
+        e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        done[dev].store(true);
+    }
+    return cudaSuccess;
+}
+
 // Launch that may start while the kernel before it on the stream is still
 // running (programmatic dependent launch): `kernel` calls pdl_wait() before
 // its first global access, so only its launch and its index arithmetic

@@ -2051,8 +2051,10 @@ int set_smem_attrs()
     return LBM_OK;
 }
 
-// once per device: the head's dynamic shared memory (two staged chunks of up
-// to 256 rows and 48 KB of weights)
+// Once per device: the most dynamic shared memory any launch of these kernels
+// takes (the limit belongs to the kernel, which other host threads use too, so
+// no launch may set it to its own size).  Head: two staged chunks of up to 256
+// rows and 48 KB of weights; lift backward: the sums of 1024 channels.
 int set_head_attrs()
 {
     static std::mutex mu;
@@ -2061,12 +2063,17 @@ int set_head_attrs()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LBM_ECUDA;
     std::lock_guard<std::mutex> lock(mu);
     if (done[dev]) return LBM_OK;
-    const void *fn[] = {(const void *)k_head<3, 1>,  (const void *)k_head<3, 2>,  (const void *)k_head<6, 1>,
-                        (const void *)k_head<6, 2>,  (const void *)k_head<12, 1>, (const void *)k_head<12, 2>,
-                        (const void *)k_head<24, 1>, (const void *)k_head<24, 2>};
-    for (const void *f : fn)
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 48 * 1024 + 2 * 256 * kHeadPitch) != cudaSuccess)
+    constexpr int head = 48 * 1024 + 2 * 256 * kHeadPitch;
+    const struct {
+        const void *fn;
+        int bytes;
+    } all[] = {{(const void *)k_head<3, 1>, head},  {(const void *)k_head<3, 2>, head},
+               {(const void *)k_head<6, 1>, head},  {(const void *)k_head<6, 2>, head},
+               {(const void *)k_head<12, 1>, head}, {(const void *)k_head<12, 2>, head},
+               {(const void *)k_head<24, 1>, head}, {(const void *)k_head<24, 2>, head},
+               {(const void *)k_lift_bwd<16>, 1024 * 17 * 4}, {(const void *)k_lift_bwd<32>, 1024 * 33 * 4}};
+    for (const auto &k : all)
+        if (cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.bytes) != cudaSuccess)
             return LBM_ECUDA;
     done[dev] = true;
     return LBM_OK;
@@ -2277,11 +2284,10 @@ int lbm_nn_lift_backward(const float *gx0, const float *feat, float *gWl, float 
     const size_t sh = sizeof(float) * std::max((size_t)per_block * F, (size_t)C * (F + 1));
     cudaStream_t s = (cudaStream_t)stream;
     // [C][F + 1] sums of 1024 channels and 32 features exceed 48 KB
-    const void *fn = F == 4 ? (const void *)k_lift_bwd<4> : F == 8 ? (const void *)k_lift_bwd<8>
-                   : F == 16 ? (const void *)k_lift_bwd<16> : (const void *)k_lift_bwd<32>;
-    if (sh > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh) != cudaSuccess)
-        return LBM_ECUDA;
+    if (sh > 48 * 1024) {
+        const int rc = set_head_attrs();
+        if (rc != LBM_OK) return rc;
+    }
     switch (F) {
     case 4: return launched(launch_pdl(k_lift_bwd<4>, dim3(blocks), threads, sh, s, gx0, feat, gWl, gbl, P, C, per_block));
     case 8: return launched(launch_pdl(k_lift_bwd<8>, dim3(blocks), threads, sh, s, gx0, feat, gWl, gbl, P, C, per_block));
