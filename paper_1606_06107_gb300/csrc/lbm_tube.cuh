@@ -4,8 +4,9 @@
 //
 // Every multiply-add is written out, no product feeds an addition directly
 // (the packed instructions are contracted even where the scalar ones are not
-// allowed to be), and the files that include this are compiled without
-// contraction, so each node's result is the same bits from either form.  Against the general kernel's expressions (k_step, contracted
+// allowed to be; vmul_alone is the exception), and the files that include this
+// are compiled without contraction, so each node's result is the same bits from
+// either form.  Against the general kernel's expressions (k_step, contracted
 // nowhere) the polynomial's coefficients are factored, mirror velocities share
 // the equilibrium of h, the upwind stencil is three multiply-adds and the
 // division by (D + n)/2 is a reciprocal product with one correction
@@ -178,11 +179,10 @@ __device__ __forceinline__ void tube_update(const TubeLattice &c, const TubeRate
     acc0 = vfma(k1(c.w[0]), a00, acc0);
     const V d0 = vfma(om, rho, vneg(acc0));
     const V d2 = vfma(om, E2_eq, vneg(acc2));
-    const V b = vmul(d2, k1(0.5f));
     const V dm = vmul(k1(0.5f), vfma(om, j, vneg(accj)));
     st(3, vfma(keep, g[3], vfma(k1(c.w[0]), a00, vsub(d0, d2))));
-    st(2, vfma(keep, g[2], moved(2, vfma(k1(c.w[1]), qm, vsub(b, dm)))));
-    st(4, vfma(keep, g[4], moved(4, vfma(k1(c.w[1]), qp, vadd(b, dm)))));
+    st(2, vfma(keep, g[2], moved(2, vfma(k1(c.w[1]), qm, vfma(k1(0.5f), d2, vneg(dm))))));
+    st(4, vfma(keep, g[4], moved(4, vfma(k1(c.w[1]), qp, vfma(k1(0.5f), d2, dm)))));
 
     // ---- rotational populations ---------------------------------------------
     if (ROT) {
