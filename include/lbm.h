@@ -298,13 +298,13 @@ int lbm_batch_get_moments(lbm_batch b, float *rho, float *u, float *T);
  * and the number of problems whose word is non-zero.  Synchronizing. */
 int lbm_batch_status(lbm_batch b, int *status, int *n_bad);
 
-/* Shape of the persistent launch: nodes a block updates at a time, two per
- * thread (`threads`: 32..1024, a multiple of 32), and resident blocks per SM
- * (0 = as many as fit; fewer keep more of each problem's state in L2).  lbm_batch_autotune times `sample_steps`
- * steps of the bound ensemble for every pair of 128/256/512/1024 nodes and
- * 1/2/4/max blocks per SM and keeps the fastest (returned through the
- * pointers, which may be NULL).  Autotuning advances the state: call
- * lbm_batch_set_macro afterwards. */
+/* Shape of the persistent launch: threads per block, a node each (`threads`:
+ * 32..1024, a multiple of 32; a run takes no more than its longest problem or
+ * the number of problems gives work to), and resident blocks per SM (0 = as
+ * many as fit).  lbm_batch_autotune times `sample_steps` steps of the bound
+ * ensemble for every pair of 128/256/512/1024 threads and 1/2/4/max blocks per
+ * SM and keeps the fastest (returned through the pointers, which may be NULL).
+ * Autotuning advances the state: call lbm_batch_set_macro afterwards. */
 int lbm_batch_set_block(lbm_batch b, int threads, int blocks_per_sm);
 int lbm_batch_autotune(lbm_batch b, int64_t sample_steps, int *threads, int *blocks_per_sm);
 

@@ -87,9 +87,10 @@ __device__ __forceinline__ Params<7> tube_params(const BatchParams &bp, const Tu
 // node by node and 15 floats apart: every population and neighbour is an
 // immediate offset from one address (a third of the instructions of the
 // population-major form were address arithmetic), and the odd pitch keeps
-// consecutive lanes on different banks.  Each thread updates two nodes at a
-// time, half a window apart, in packed arithmetic (f32x2), with a block
-// barrier between steps and three copies of an end's node beyond it.
+// consecutive lanes on different banks.  A thread updates one node at a time,
+// with a block barrier between steps; the new state is stored after the last
+// load, and an end's thread stores its node's three copies beyond the end from
+// registers.
 //
 // A problem that fits (kWindow nodes, 108 KB: two blocks an SM) is loaded once
 // and stored after its last step.  A longer one goes through the two global
@@ -99,12 +100,17 @@ __device__ __forceinline__ Params<7> tube_params(const BatchParams &bp, const Tu
 // exactly what whole steps give; the nodes beside it go wrong from the
 // window's ends inwards and are dropped.  Against one pass over the global
 // buffers per step this reads and writes L2 once in sixteen steps, for 8-12 %
-// more nodes.  Bound by shared-memory reads (57 % of the LSU's
-// rate at 1024 windows of 384 nodes) and the barriers between steps: 1024 x
-// 384 nodes, 32 FD steps 180 us (261 with one node per thread, population by
-// population); 1024 tubes of 256-8192 nodes, 50 FD steps 3.43 ms (6.53 through
-// the global buffers).  Passes of 8 / 12 / 16 steps 3.66 / 3.52 / 3.43 ms;
-// windows of 448 nodes 3.84; 256 / 1024 nodes at a time 4.57 / 4.38.
+// more nodes.
+//
+// Bound by shared-memory reads and the barriers between steps.  One node a
+// thread against two in packed arithmetic (f32x2, half a window apart), 32 FD
+// steps: 1024 tubes of 4096 nodes 1.78 / 2.01 ms, of 640 285 / 335 us, of 384 179
+// / 172, of 100-150 83 / 102; 152 tubes of 384 41 / 54, one of 100-150 30 / 45: a
+// step of a short problem is one node's chain of instructions.  Copying the end's
+// node through shared memory, value by value, made that chain 0.5 us longer.
+// 1024 tubes of 256-8192 nodes, 50 FD steps 3.12 ms (6.53 through the global
+// buffers); passes of 8 / 12 / 16 steps and windows of 448 / 896 nodes, two nodes
+// a thread: 3.66 / 3.52 / 3.43 and 3.84 / 3.43.
 constexpr int kNodePitch = 15;
 #ifndef LBM_BATCH_WINDOW
 #define LBM_BATCH_WINDOW 896
@@ -118,10 +124,8 @@ constexpr int kPassSteps = LBM_BATCH_PASS;
 #define LBM_BATCH_THREADS 512
 #endif
 
-// (768: at most 512 threads run; the bound keeps the registers at 80, so that
-// four blocks of 192 threads fit an SM)
 template <int MODE>
-__global__ void __launch_bounds__(768) k_batch_run(const BatchParams bp, const TubeLattice lat, int nodes)
+__global__ void __launch_bounds__(1024) k_batch_run(const BatchParams bp, const TubeLattice lat, int nodes)
 {
     extern __shared__ float sm[];  // [2][nodes][kNodePitch]
     __shared__ int claim;
@@ -165,47 +169,33 @@ __global__ void __launch_bounds__(768) k_batch_run(const BatchParams bp, const T
                 }
                 __syncthreads();
                 const bool left = w0 == 0, right = w1 == d.len;
-                const int half = (n + 1) / 2;
+                const int watch_lo = max(i0, d.watch_lo), watch_hi = min(i1, d.watch_hi);
                 for (int64_t s = 0; s < steps; ++s) {
-                    for (int l = threadIdx.x; l < half; l += blockDim.x) {
-                        const bool two = l + half < n;
-                        const int l1 = two ? l + half : l;
-                        const float *m0 = a + (l + 3) * kNodePitch, *m1 = a + (l1 + 3) * kNodePitch;
-                        float *o0 = c + (l + 3) * kNodePitch, *o1 = c + (l1 + 3) * kNodePitch;
-                        F2 rho, T;
-                        tube_update<true, MODE, F2>(
-                            lat, rates,
-                            [&](int pop, int dx) { return f2(m0[dx * kNodePitch + pop], m1[dx * kNodePitch + pop]); },
-                            [&](F2 ux) {
-                                const int p0 = lo(ux) >= 0.f ? -kNodePitch : kNodePitch;
-                                const int p1 = hi(ux) >= 0.f ? -kNodePitch : kNodePitch;
-                                const float *u0 = m0 + p0, *v0 = m0 + 2 * p0, *d0 = m0 - p0;
-                                const float *u1 = m1 + p1, *v1 = m1 + 2 * p1, *d1 = m1 - p1;
-                                return [=](int j, int kk) {
-                                    return kk == 2 ? f2(v0[7 + j], v1[7 + j])
-                                                   : kk == 1 ? f2(u0[7 + j], u1[7 + j]) : f2(d0[7 + j], d1[7 + j]);
-                                };
+                    for (int l = threadIdx.x; l < n; l += blockDim.x) {
+                        const float *me = a + (l + 3) * kNodePitch;
+                        float out[14], rho, T;
+                        tube_update<true, MODE>(
+                            lat, rates, [&](int pop, int dx) { return me[dx * kNodePitch + pop]; },
+                            [&](float ux) {
+                                const int up = ux >= 0.f ? -kNodePitch : kNodePitch;
+                                const float *u1 = me + up, *u2 = me + 2 * up, *d1 = me - up;
+                                return [u1, u2, d1](int j, int kk) { return (kk == 2 ? u2 : kk == 1 ? u1 : d1)[7 + j]; };
                             },
-                            [&](int pop, F2 v) {
-                                o0[pop] = lo(v);
-                                if (two) o1[pop] = hi(v);
-                            },
-                            rho, T);
-                        const int x0 = w0 + l, x1 = w0 + l1;
-                        const int lo_w = max(i0, d.watch_lo), hi_w = min(i1, d.watch_hi);
-                        if ((tube_bad(lo(rho), lo(T)) && x0 >= lo_w && x0 < hi_w) ||
-                            (tube_bad(hi(rho), hi(T)) && x1 >= lo_w && x1 < hi_w))
-                            atomicOr(bp.status + k, 1);
+                            out, rho, T);
+                        if (tube_bad(rho, T) && w0 + l >= watch_lo && w0 + l < watch_hi) atomicOr(bp.status + k, 1);
+                        auto put = [&](int at) {
+#pragma unroll
+                            for (int i = 0; i < 14; ++i) c[at * kNodePitch + i] = out[i];
+                        };
+                        put(l + 3);
                         // the copies beyond the problem's ends
                         if (left && l == 0) {
 #pragma unroll 1
-                            for (int g = 0; g < 3; ++g)
-                                for (int i = 0; i < 14; ++i) c[g * kNodePitch + i] = o0[i];
+                            for (int g = 0; g < 3; ++g) put(g);
                         }
-                        if (right && l1 == n - 1) {
+                        if (right && l == n - 1) {
 #pragma unroll 1
-                            for (int g = 0; g < 3; ++g)
-                                for (int i = 0; i < 14; ++i) c[(n + 3 + g) * kNodePitch + i] = o1[i];
+                            for (int g = 0; g < 3; ++g) put(n + 3 + g);
                         }
                     }
                     float *t = a;
@@ -283,7 +273,7 @@ struct lbm_batch_ctx {
     char *work = nullptr;
     cudaStream_t stream = nullptr;
     int cur = 0;
-    int threads = LBM_BATCH_THREADS;  // nodes a block updates at a time, two a thread
+    int threads = LBM_BATCH_THREADS;  // threads per block at most, a node each
     int blocks_per_sm = 0;            // resident blocks per SM of the persistent grid (0 = max)
     int64_t launches = 0;
     std::string err;
@@ -335,23 +325,34 @@ BatchParams batch_params(const lbm_batch_ctx *b, long long steps)
 
 bool aligned(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
 
-// The persistent kernel of a run, its threads (two nodes each) and its
-// dynamic shared memory.
+// The persistent kernel of a run, its threads and its dynamic shared memory.
 const void *run_kernel(const lbm_batch_ctx *b)
 {
     return (b->mode == LBM_MODE_FD) ? (const void *)lbm::k_batch_run<1> : (const void *)lbm::k_batch_run<0>;
 }
-int run_threads(int threads) { return std::max(32, (threads / 2 + 31) / 32 * 32); }
+// No more threads than a window has nodes: the others would take registers from
+// other blocks (1024 tubes of 100-150 nodes, two nodes a thread: 108 us with as
+// many as needed, 145 with 256).  Windows of 257 to 512 nodes, from three problems per SM on: 256
+// threads, which four blocks an SM can have: 600 / 1024 / 3000 problems of 450-512
+// nodes 127 / 217 / 571 us against 164 / 229 / 618 with a node a thread; 300 / 450
+// problems 76 / 103 against 75 / 102.
+int run_threads(const lbm_batch_ctx *b, int threads, int sms)
+{
+    const int nodes = (b->window - 6 + 31) / 32 * 32;
+    const int most = nodes > 256 && nodes <= 512 && b->count > 3 * sms ? 256 : nodes;
+    return std::min(threads, most);
+}
 int run_smem(const lbm_batch_ctx *b) { return (int)sizeof(float) * 2 * lbm::kNodePitch * b->window; }
 
-// Resident-block grid of the persistent kernel for `threads` per block.
-cudaError_t persistent_grid(const lbm_batch_ctx *b, int threads, int bps, int *grid)
+// Threads per block and grid of the persistent kernel.
+cudaError_t persistent_grid(const lbm_batch_ctx *b, int threads, int bps, int *block, int *grid)
 {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const void *fn = run_kernel(b);
+    *block = run_threads(b, threads, sms);
     // (the limit is a property of the kernel, which other ensembles share: the
     // largest any of them takes)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -359,19 +360,21 @@ cudaError_t persistent_grid(const lbm_batch_ctx *b, int threads, int bps, int *g
     if (e == cudaSuccess)  // all of L1 as shared memory: the kernel reads nothing twice through it
         e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, run_threads(threads), run_smem(b));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, *block, run_smem(b));
     if (e != cudaSuccess) return e;
     per_sm = std::max(1, per_sm);
     if (bps > 0) per_sm = std::min(per_sm, bps);
-    *grid = per_sm * sms;
+    // (a block per problem at most: more would claim unevenly, several problems
+    // on some SMs while others have none)
+    *grid = std::min(per_sm * sms, b->count);
     return cudaSuccess;
 }
 
 // The graph of one run: reset the claim counter, then the persistent kernel.
 int build_graph(lbm_batch b, long long steps, cudaGraphExec_t *exec)
 {
-    int grid = 0;
-    cudaError_t e = persistent_grid(b, b->threads, b->blocks_per_sm, &grid);
+    int block = 0, grid = 0;
+    cudaError_t e = persistent_grid(b, b->threads, b->blocks_per_sm, &block, &grid);
     if (e != cudaSuccess) return bcuda(b, e, "occupancy query");
     cudaGraph_t g = nullptr;
     e = cudaGraphCreate(&g, 0);
@@ -392,7 +395,7 @@ int build_graph(lbm_batch b, long long steps, cudaGraphExec_t *exec)
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void *>(run_kernel(b));
     kp.gridDim = dim3(grid);
-    kp.blockDim = dim3(run_threads(b->threads));
+    kp.blockDim = dim3(block);
     kp.sharedMemBytes = (unsigned)run_smem(b);
     kp.kernelParams = args;
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&n_run, g, &n_reset, 1, &kp);

@@ -45,8 +45,8 @@ template <bool ROT, int MODE> __global__ void __launch_bounds__(kBlockX) k_tube_
     for (int k = 0; k < 7; ++k) o[k] = bc_wrap(x + k - 3, p.X, p.bc);
     pdl_wait();
     pdl_trigger();
-    float out[ROT ? 14 : 7], rho, T;  // stored together: no load waits for a store
-    tube_update<ROT, MODE, float>(
+    float out[ROT ? 14 : 7], rho, T;
+    tube_update<ROT, MODE>(
         p.lat, p.rates, [&](int pop, int d) { return __ldca(p.src + ((uint32_t)pop * (uint32_t)p.S + (uint32_t)o[3 + d])); },
         [&](float ux) {
             const bool pos = ux >= 0.f;
@@ -55,7 +55,7 @@ template <bool ROT, int MODE> __global__ void __launch_bounds__(kBlockX) k_tube_
                 return __ldca(p.src + ((uint32_t)(7 + j) * (uint32_t)p.S + (uint32_t)(k == 2 ? u2 : k == 1 ? u1 : d1)));
             };
         },
-        [&](int pop, float v) { out[pop] = v; }, rho, T);
+        out, rho, T);
 #pragma unroll
     for (int i = 0; i < (ROT ? 14 : 7); ++i) p.dst[(uint32_t)i * (uint32_t)p.S + (uint32_t)x] = out[i];
     if (tube_bad(rho, T)) atomicOr(p.status, 1);
@@ -106,14 +106,14 @@ __global__ void __launch_bounds__(MAXT) k_tube_steps(const TubeParams p, int64_t
         if (l < n) {
             const float *me = a + (l + 3) * kNodePitch;
             float out[POPS], rho, T;
-            tube_update<ROT, MODE, float>(
+            tube_update<ROT, MODE>(
                 p.lat, p.rates, [&](int pop, int d) { return me[d * kNodePitch + pop]; },
                 [&](float ux) {
                     const int up = ux >= 0.f ? -kNodePitch : kNodePitch;
                     const float *u1 = me + up, *u2 = me + 2 * up, *d1 = me - up;
                     return [u1, u2, d1](int j, int k) { return (k == 2 ? u2 : k == 1 ? u1 : d1)[7 + j]; };
                 },
-                [&](int pop, float v) { out[pop] = v; }, rho, T);
+                out, rho, T);
             if (tube_bad(rho, T)) atomicOr(p.status, 1);
             auto put = [&](float *base, int at) {
 #pragma unroll

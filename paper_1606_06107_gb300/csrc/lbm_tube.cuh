@@ -1,18 +1,15 @@
 // The node update of the one-dimensional problems in float storage (D1Q7 +
-// D1Q7): one node per thread (V = float: single steps and the many-step
-// kernel, lbm_d1q7.cu) or two (V = F2: the ensemble, lbm_batch.cu).
+// D1Q7), one node per thread: single steps and the many-step kernel
+// (lbm_d1q7.cu) and the ensemble (lbm_batch.cu).
 //
-// Every multiply-add is written out, no product feeds an addition directly
-// (the packed instructions are contracted even where the scalar ones are not
-// allowed to be; vmul_alone is the exception), and the files that include this
-// are compiled without contraction, so each node's result is the same bits from
-// either form.  Against the general kernel's expressions (k_step, contracted
-// nowhere) the polynomial's coefficients are factored, mirror velocities share
-// the equilibrium of h, the upwind stencil is three multiply-adds and the
-// division by (D + n)/2 is a reciprocal product with one correction
-// (Markstein, IBM J. Res. Dev. 34(1), 1990: correctly rounded, since 1/cT is):
-// about 220 operations per node instead of 380 (1000 nodes, FD: 0.75 us per step
-// in one launch, 1.04 with the general expressions).
+// Every multiply-add is written out and the files that include this are
+// compiled without contraction, so all of them give the same bits.  Against the
+// general kernel's expressions (k_step) the polynomial's coefficients are
+// factored, mirror velocities share the equilibrium of h, the upwind stencil is
+// three multiply-adds and the division by (D + n)/2 is a reciprocal product with
+// one correction (Markstein, IBM J. Res. Dev. 34(1), 1990: correctly rounded,
+// since 1/cT is): about 220 operations per node instead of 380 (1000 nodes, FD:
+// 0.75 us per step in one launch, 1.04 with the general expressions).
 //
 // The order of the sums is part of the accuracy, because a rounding that recurs
 // every step adds up over thousands of them: a new population is
@@ -22,37 +19,11 @@
 // that of the general expressions, geometric mean of forty 1000-node FD tubes,
 // n = 4, 2000 steps: rho 0.91, u 0.88, T 1.04 (tau 0.7-1), 0.82, 0.70, 1.08 (tau
 // 2/3); 200 steps 0.95, 0.86, 0.97.  With fma(convection, .., fma(1 - omega, old,
-// omega eq)) and half the moment doubled 1.69, 1.51, 2.08 and 1.69, 1.45, 2.85:
-// 1-2 % faster in the ensemble.
+// omega eq)) and half the moment doubled 1.69, 1.51, 2.08 and 1.69, 1.45, 2.85.
 #pragma once
 #include "lbm_step.cuh"
 
 namespace lbm {
-
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
-// a product that an addition follows, in a form that cannot be contracted
-__device__ __forceinline__ float vmul_alone(float a, float b) { return a * b; }
-__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
-__device__ __forceinline__ float vsub(float a, float b) { return a - b; }
-__device__ __forceinline__ float vneg(float a) { return -a; }
-__device__ __forceinline__ float vabs(float a) { return fabsf(a); }
-__device__ __forceinline__ float vrcp(float a) { return __frcp_rn(a); }
-__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return fma2(a, b, c); }
-__device__ __forceinline__ F2 vmul(F2 a, F2 b) { return mul2(a, b); }
-__device__ __forceinline__ F2 vmul_alone(F2 a, F2 b) { return f2(__fmul_rn(lo(a), lo(b)), __fmul_rn(hi(a), hi(b))); }
-__device__ __forceinline__ F2 vadd(F2 a, F2 b) { return add2(a, b); }
-__device__ __forceinline__ F2 vsub(F2 a, F2 b) { return sub2(a, b); }
-__device__ __forceinline__ F2 vneg(F2 a) { return neg2(a); }
-__device__ __forceinline__ F2 vabs(F2 a) { return F2{a.v & 0x7fffffff7fffffffull}; }
-__device__ __forceinline__ F2 vrcp(F2 a) { return f2(__frcp_rn(lo(a)), __frcp_rn(hi(a))); }
-template <typename V> struct Splat;
-template <> struct Splat<float> {
-    __device__ __forceinline__ static float of(float s) { return s; }
-};
-template <> struct Splat<F2> {
-    __device__ __forceinline__ static F2 of(float s) { return f2(s); }
-};
 
 // Constants of the lattice and the transport, by |e| = 0..3.
 struct TubeLattice {
@@ -93,16 +64,17 @@ __host__ __device__ __forceinline__ TubeRates tube_rates(float omega, float cT, 
     return TubeRates{omega, 1.0f - omega, cT, 1.0f / cT, half_n};
 }
 
-// One step of one node (or two).  ld(pop, d): population pop (g_0..g_6, then
-// h_0..h_6) at node x + d.  stencil(ux) fixes the upwind side of h and
-// returns a loader up(j, k): h_j two (k = 2) or one (1) nodes upwind, or one
-// downwind (-1).  st(pop, v) stores.  rho and T are returned for the status.
-template <bool ROT, int MODE, typename V, typename Ld, typename Stencil, typename St>
+// One step of one node.  ld(pop, d): population pop (g_0..g_6, then h_0..h_6)
+// at node x + d.  stencil(ux) fixes the upwind side of h and returns a loader
+// up(j, k): h_j two (k = 2) or one (1) nodes upwind, or one downwind (-1).  The
+// new populations come back in `out`, for the caller to store together (a load
+// does not move above a store that might be to the same address); rho and T
+// are returned for the status.
+template <bool ROT, int MODE, typename Ld, typename Stencil>
 __device__ __forceinline__ void tube_update(const TubeLattice &c, const TubeRates &q, Ld &&ld, Stencil &&stencil,
-                                            St &&st, V &rho_out, V &T_out)
+                                            float (&out)[ROT ? 14 : 7], float &rho_out, float &T_out)
 {
-    auto k1 = [](float s) { return Splat<V>::of(s); };
-    V g[7], h[7];
+    float g[7], h[7];
 #pragma unroll
     for (int i = 0; i < 7; ++i) g[i] = ld(i, MODE == 0 ? 3 - i : 0);
     if (ROT) {
@@ -110,108 +82,97 @@ __device__ __forceinline__ void tube_update(const TubeLattice &c, const TubeRate
         for (int j = 0; j < 7; ++j) h[j] = ld(7 + j, 0);
     }
     // ---- moments (Sec. V steps 3-4, Eq. T), opposite velocities first -------
-    V rho = g[3], j = k1(0.f), e2 = k1(0.f), R2 = k1(0.f);
+    float rho = g[3], j = 0.f, e2 = 0.f, R2 = 0.f;
 #pragma unroll
     for (int k = 1; k <= 3; ++k) {
-        const V s = vadd(g[3 + k], g[3 - k]);
-        rho = vadd(rho, s);
-        j = vfma(k1((float)k), vsub(g[3 + k], g[3 - k]), j);
-        e2 = vfma(k1((float)(k * k)), s, e2);
-        if (ROT) R2 = vfma(k1((float)(k * k)), vadd(h[3 + k], h[3 - k]), R2);
+        const float s = g[3 + k] + g[3 - k];
+        rho += s;
+        j = fmaf((float)k, g[3 + k] - g[3 - k], j);
+        e2 = fmaf((float)(k * k), s, e2);
+        if (ROT) R2 = fmaf((float)(k * k), h[3 + k] + h[3 - k], R2);
     }
-    const V inv_rho = vrcp(rho);
-    const V ux = vmul(vmul(k1(c.r), j), inv_rho);
-    const V j2 = vmul(j, j);
-    V e = vmul(vmul(k1(0.5f), vfma(vneg(j2), inv_rho, e2)), inv_rho);
-    if (ROT) e = vfma(k1(q.half_n), R2, e);
+    const float inv_rho = __frcp_rn(rho);
+    const float ux = c.r * j * inv_rho, j2 = j * j;
+    float e = 0.5f * fmaf(-j2, inv_rho, e2) * inv_rho;
+    if (ROT) e = fmaf(q.half_n, R2, e);
     // e / cT: the quotient's residual corrects the reciprocal product
-    V T_lat = vmul(e, k1(q.inv_cT));
-    T_lat = vfma(vfma(vneg(T_lat), k1(q.cT), e), k1(q.inv_cT), T_lat);
-    const V E2_eq = vfma(rho, T_lat, vmul(j2, inv_rho));  // rho (u^2 + T) / r^2
+    float T_lat = e * q.inv_cT;
+    T_lat = fmaf(fmaf(-T_lat, q.cT, e), q.inv_cT, T_lat);
+    const float E2_eq = fmaf(rho, T_lat, j2 * inv_rho);  // rho (u^2 + T) / r^2
     rho_out = rho;
-    T_out = vmul(k1(c.r2), T_lat);
+    T_out = c.r2 * T_lat;
 
     // ---- coefficients of omega rho g^eq / w (eq_coef at D = 1) --------------
-    const V t = vfma(k1(c.r2), T_lat, k1(-1.0f)), u2 = vmul(ux, ux), om = k1(q.omega), keep = k1(q.keep);
-    const V scale = vmul(om, rho), st1 = vmul(scale, t);
-    const V a00 = vmul(scale, vfma(u2, vfma(k1(0.75f), t, vfma(k1(0.125f), u2, k1(-0.5f))),
-                                   vfma(t, vfma(k1(0.375f), t, k1(-0.5f)), k1(1.0f))));
-    const V a01 = vmul(st1, vfma(k1(-0.75f), t, vfma(k1(-0.25f), u2, k1(0.5f))));
-    const V a02 = vmul(k1(0.125f), vmul(st1, t));
-    const V a10 = vmul(scale, vfma(k1(-1.5f), t, vfma(k1(-0.5f), u2, k1(1.0f))));
-    const V a11 = vmul(k1(0.5f), st1);
-    const V a20 = vmul(scale, vfma(k1(-1.25f), t, vfma(k1(-0.25f), u2, k1(0.5f))));
-    const V a21 = vmul(k1(0.25f), st1);
-    const V k6 = vmul(k1(1.0f / 6.0f), scale), k24 = vmul(k1(1.0f / 24.0f), scale);
-    const V ru = vmul(k1(c.r), ux);
+    const float t = fmaf(c.r2, T_lat, -1.0f), u2 = ux * ux, om = q.omega, keep = q.keep;
+    const float scale = om * rho, st = scale * t;
+    const float a00 = scale * fmaf(u2, fmaf(0.75f, t, fmaf(0.125f, u2, -0.5f)), fmaf(t, fmaf(0.375f, t, -0.5f), 1.0f));
+    const float a01 = st * fmaf(-0.75f, t, fmaf(-0.25f, u2, 0.5f)), a02 = 0.125f * (st * t);
+    const float a10 = scale * fmaf(-1.5f, t, fmaf(-0.5f, u2, 1.0f)), a11 = 0.5f * st;
+    const float a20 = scale * fmaf(-1.25f, t, fmaf(-0.25f, u2, 0.5f)), a21 = 0.25f * st;
+    const float k6 = (1.0f / 6.0f) * scale, k24 = (1.0f / 24.0f) * scale;
+    const float ru = c.r * ux;
 
     // ---- collision and transport of g ---------------------------------------
-    // the transport term of population i subtracted from v
-    auto moved = [&](int i, V v) {
-        if (MODE == 0) return v;
+    // (1 - omega) g_i + v less the transport term
+    auto put = [&](int i, float v) {
         const int ei = i - 3, m = ei < 0 ? -ei : ei, up = ei > 0 ? -1 : 1;
-        if (m == 0) return v;
-        V x = vfma(k1(-6.0f), ld(i, up), ld(i, 2 * up));
-        x = vfma(k1(3.0f), g[i], x);
-        x = vfma(k1(2.0f), ld(i, -up), x);
-        return vfma(k1(-c.ce[m]), x, v);
+        if (MODE == 1 && m != 0) {
+            float x = fmaf(-6.0f, ld(i, up), ld(i, 2 * up));
+            x = fmaf(3.0f, g[i], x);
+            x = fmaf(2.0f, ld(i, -up), x);
+            v = fmaf(-c.ce[m], x, v);
+        }
+        out[i] = fmaf(keep, g[i], v);
     };
-    V acc0 = k1(0.f), acc2 = k1(0.f), accj = k1(0.f), qm = k1(0.f), qp = k1(0.f);
+    float acc0 = 0.f, acc2 = 0.f, accj = 0.f, qm = 0.f, qp = 0.f;
 #pragma unroll
     for (int m = 3; m >= 1; --m) {
-        const V s = k1(c.s[m]), cu = vmul(k1((float)m), ru);
-        const V A0 = vfma(s, vfma(s, a02, a01), a00), A1 = vfma(s, a11, a10), A2 = vfma(s, a21, a20);
-        const V c2 = vmul(cu, cu);
-        const V E = vfma(c2, vfma(c2, k24, A2), A0), O = vfma(c2, k6, A1);  // P(+-c) = E +- c O
-        const V w = k1(c.w[m]);
-        const V pp = vfma(cu, O, E), pm = vfma(vneg(cu), O, E), sum = vadd(pp, pm);
-        acc0 = vfma(w, sum, acc0);
-        acc2 = vfma(k1(c.w2[m]), sum, acc2);
-        accj = vfma(k1(c.w1[m]), vsub(pp, pm), accj);
-        if (m == 1) {  // stored last, with the corrections
+        const float s = c.s[m], cu = (float)m * ru, c2 = cu * cu;
+        const float A0 = fmaf(s, fmaf(s, a02, a01), a00), A1 = fmaf(s, a11, a10), A2 = fmaf(s, a21, a20);
+        const float E = fmaf(c2, fmaf(c2, k24, A2), A0), O = fmaf(c2, k6, A1);  // P(+-c) = E +- c O
+        const float w = c.w[m], pp = fmaf(cu, O, E), pm = fmaf(-cu, O, E), sum = pp + pm;
+        acc0 = fmaf(w, sum, acc0);
+        acc2 = fmaf(c.w2[m], sum, acc2);
+        accj = fmaf(c.w1[m], pp - pm, accj);
+        if (m == 1) {  // last, with the corrections
             qm = pm;
             qp = pp;
         } else {
-            st(3 - m, vfma(keep, g[3 - m], moved(3 - m, vmul(w, pm))));
-            st(3 + m, vfma(keep, g[3 + m], moved(3 + m, vmul(w, pp))));
+            put(3 - m, w * pm);
+            put(3 + m, w * pp);
         }
     }
-    acc0 = vfma(k1(c.w[0]), a00, acc0);
-    const V d0 = vfma(om, rho, vneg(acc0));
-    const V d2 = vfma(om, E2_eq, vneg(acc2));
-    const V dm = vmul(k1(0.5f), vfma(om, j, vneg(accj)));
-    st(3, vfma(keep, g[3], vfma(k1(c.w[0]), a00, vsub(d0, d2))));
-    st(2, vfma(keep, g[2], moved(2, vfma(k1(c.w[1]), qm, vfma(k1(0.5f), d2, vneg(dm))))));
-    st(4, vfma(keep, g[4], moved(4, vfma(k1(c.w[1]), qp, vfma(k1(0.5f), d2, dm)))));
+    acc0 = fmaf(c.w[0], a00, acc0);
+    const float d0 = fmaf(om, rho, -acc0);
+    const float d2 = fmaf(om, E2_eq, -acc2);
+    const float dm = 0.5f * fmaf(om, j, -accj);
+    put(3, fmaf(c.w[0], a00, d0 - d2));
+    put(2, fmaf(c.w[1], qm, fmaf(0.5f, d2, -dm)));
+    put(4, fmaf(c.w[1], qp, fmaf(0.5f, d2, dm)));
 
     // ---- rotational populations ---------------------------------------------
     if (ROT) {
         // h^eq with its moments put right (heq_node): mirror entries are equal,
         // their contributions to the second moment still added one by one
-        V eq[4];
+        float eq[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) eq[k] = vfma(t, vfma(t, k1(c.hb[k]), k1(c.ha[k])), k1(1.0f));
-        const V e1 = vmul_alone(k1(c.w[1]), eq[1]), e2w = vmul(k1(c.w[2]), eq[2]), e3 = vmul(k1(c.w[3]), eq[3]);
-        V m2 = vfma(k1(4.0f), e2w, vmul(k1(9.0f), e3));
-        m2 = vfma(k1(9.0f), e3, vfma(k1(4.0f), e2w, vadd(vadd(m2, e1), e1)));
-        const V d = vsub(T_lat, m2);
-        const V half0 = vadd(e1, vfma(k1(c.w[2]), eq[2], e3));
-        eq[0] = vfma(k1(c.w[0]), eq[0], vsub(vfma(k1(-2.0f), half0, vfma(k1(-c.w[0]), eq[0], k1(1.0f))), d));
-        eq[1] = vfma(k1(0.5f), d, e1);
-        eq[2] = e2w;
-        eq[3] = e3;
-        const V anu = vneg(vabs(vmul(ux, k1(c.nu6))));
+        for (int k = 0; k < 4; ++k) eq[k] = fmaf(t, fmaf(t, c.hb[k], c.ha[k]), 1.0f);
+        const float q1 = c.w[1] * eq[1], q2 = c.w[2] * eq[2], q3 = c.w[3] * eq[3];
+        const float m2 = fmaf(9.0f, q3, fmaf(4.0f, q2, fmaf(4.0f, q2, 9.0f * q3) + q1 + q1));
+        const float d = T_lat - m2;
+        const float half0 = q1 + fmaf(c.w[2], eq[2], q3);
+        eq[0] = fmaf(c.w[0], eq[0], fmaf(-2.0f, half0, fmaf(-c.w[0], eq[0], 1.0f)) - d);
+        eq[1] = fmaf(0.5f, d, q1);
+        eq[2] = q2;
+        eq[3] = q3;
+        const float anu = -fabsf(ux * c.nu6);
         auto up = stencil(ux);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-#pragma unroll
-            for (int sgn = 0; sgn < (k ? 2 : 1); ++sgn) {
-                const int jj7 = sgn ? 3 + k : 3 - k;
-                V x = vfma(k1(-6.0f), up(jj7, 1), up(jj7, 2));
-                x = vfma(k1(3.0f), h[jj7], x);
-                x = vfma(k1(2.0f), up(jj7, -1), x);
-                st(7 + jj7, vfma(keep, h[jj7], vfma(om, eq[k], vmul(anu, x))));
-            }
+        for (int j7 = 0; j7 < 7; ++j7) {
+            float x = fmaf(-6.0f, up(j7, 1), up(j7, 2));
+            x = fmaf(3.0f, h[j7], x);
+            x = fmaf(2.0f, up(j7, -1), x);
+            out[7 + j7] = fmaf(keep, h[j7], fmaf(om, eq[j7 < 3 ? 3 - j7 : j7 - 3], anu * x));
         }
     }
 }

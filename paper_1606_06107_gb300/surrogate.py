@@ -520,11 +520,11 @@ def fallback_windows(L: int, width: int, margin: int):
 
 
 def _latency_block(length: int) -> int:
-    """Nodes a block updates at a time (two per thread) in an ensemble run
-    whose time is one problem's latency (a few problems, or one wave of short
-    ones): the whole problem, up to 1024.  The ensemble kernel steps a problem
-    with one block, so fewer would make each thread update several pairs in
-    turn per step."""
+    """Threads per block of an ensemble run whose time is one problem's latency
+    (a few problems, or one wave of short ones): one per node, up to 1024.
+    The ensemble kernel steps a problem with one block, so fewer would make
+    each thread update several nodes in turn per step (one 4096-node tube, 32
+    FD steps: 0.29 ms at 1024 threads, 0.37 at 256)."""
     return int(min(1024, max(32, -(-length // 32) * 32)))
 
 
