@@ -858,8 +858,9 @@ __global__ void __launch_bounds__(kBlockX, MINB) k_step(const Params<Lattice<LAT
 // Bound by the stores' bandwidth in float (229 us, 940 MB at 2048^2: 0.60 of
 // the copy bandwidth) and by issue in half (150 us; D3Q343 4.39 ms).
 // A periodic axis is a bijection (one y per population); on a copy axis the
-// edge nodes also own the y whose y + e_i the clamp brings back to them (the
-// loop over ranges at the end) and nodes within three of an edge may own none.
+// edge nodes also own the y whose y + e_i the clamp brings back to them
+// (init_spread, in threads of their own) and nodes within three of an edge may
+// own none.
 
 // Destinations lo..hi (none if lo > hi) of a node at x with velocity e on an
 // axis of n nodes: all y with bc(y + e) = x.
@@ -882,6 +883,68 @@ __host__ __device__ __forceinline__ PreImage preimage(int x, int e, int n, int b
     return r;
 }
 
+// A node's initial fields and the coefficients of its equilibrium.
+struct InitSource {
+    int64_t node;
+    float rho, T, ux, uy, uz;
+    EqCoef k;
+};
+template <int LAT, typename ST>
+__device__ __forceinline__ InitSource init_source(const Params<Lattice<LAT>::Q, ST> &p, int x, int y, int z)
+{
+    constexpr int D = Lattice<LAT>::D;
+    InitSource n;
+    n.node = ((int64_t)z * p.Y + y) * p.X + x;
+    n.rho = p.in0[n.node], n.T = p.in2[n.node];
+    n.ux = p.in1[n.node];
+    n.uy = (D >= 2) ? p.in1[p.N + n.node] : 0.f;
+    n.uz = (D >= 3) ? p.in1[2 * p.N + n.node] : 0.f;
+    n.k = eq_coef<D>(n.T, n.ux * n.ux + n.uy * n.uy + n.uz * n.uz, n.rho);
+    return n;
+}
+// The record of node `at` (per-node reference storage), from its own fields.
+template <int LAT, typename ST>
+__device__ __forceinline__ float4 init_record(const Params<Lattice<LAT>::Q, ST> &p, int64_t at)
+{
+    const float r0 = p.in0[at];
+    return make_float4(r0 - 1.0f, 0.5f * (r0 * (p.in2[at] - 1.0f)), r0 * (p.r * p.in1[at]),
+                       (Lattice<LAT>::D >= 2) ? r0 * (p.r * p.in1[p.N + at]) : 0.f);
+}
+// Population i at the destination (dx, dy, dz).
+template <int LAT, typename ST>
+__device__ __forceinline__ void init_put(const Params<Lattice<LAT>::Q, ST> &p, int i, int dx, int dy, int dz, float v)
+{
+    const int off = (dz * p.Y + dy) * p.pitch + dx;
+    if constexpr (NodeRef<ST>::value)
+        st_ref(p, i, off, v, init_record<LAT>(p, ((int64_t)dz * p.Y + dy) * p.X + dx));
+    else st(p, i, off, v);
+}
+// The further destinations of population i, velocity (ex, ey, ez), of a node on
+// a copy axis's end: all but the one that init_node writes.
+template <int LAT, typename ST>
+__device__ __forceinline__ void init_spread(const Params<Lattice<LAT>::Q, ST> &p, const InitSource &n, int x, int y,
+                                            int z, int i, int ex, int ey, int ez)
+{
+    constexpr int D = Lattice<LAT>::D;
+    auto out = [](int x, int e, int n, int bc) { return bc != 0 && ((x == 0 && e < 0) || (x == n - 1 && e > 0)); };
+    if (!(out(x, ex, p.X, p.bc0) || (D >= 2 && out(y, ey, p.Y, p.bc1)) || (D >= 3 && out(z, ez, p.Z, p.bc2)))) return;
+    const PreImage rx = preimage(x, ex, p.X, p.bc0);
+    const PreImage ry = (D >= 2) ? preimage(y, ey, p.Y, p.bc1) : PreImage{0, 0};
+    const PreImage rz = (D >= 3) ? preimage(z, ez, p.Z, p.bc2) : PreImage{0, 0};
+    const float c = p.r * ((float)ex * n.ux + (float)ey * n.uy + (float)ez * n.uz);
+    const float v = p.w[i] * eq_single(n.k, c, p.r2 * (float)(ex * ex + ey * ey + ez * ez));
+#pragma unroll 1
+    for (int dz = rz.lo; dz <= rz.hi; ++dz)
+#pragma unroll 1
+        for (int dy = ry.lo; dy <= ry.hi; ++dy)
+#pragma unroll 1
+            for (int dx = rx.lo; dx <= rx.hi; ++dx) {
+                const bool own = (p.bc0 == 0 || dx == x - ex) && (D < 2 || p.bc1 == 0 || dy == y - ey) &&
+                                 (D < 3 || p.bc2 == 0 || dz == z - ez);
+                if (!own) init_put<LAT>(p, i, dx, dy, dz, v);
+            }
+}
+
 template <int LAT, bool ROT, int MODE, typename ST>
 __device__ __forceinline__ void init_node(const Params<Lattice<LAT>::Q, ST> &p, int x, int y, int z)
 {
@@ -889,24 +952,10 @@ __device__ __forceinline__ void init_node(const Params<Lattice<LAT>::Q, ST> &p, 
     constexpr int Q = L::Q, D = L::D;
     constexpr bool is_node = NodeRef<ST>::value;
     const int self = (z * p.Y + y) * p.pitch + x;
-    const int64_t node = ((int64_t)z * p.Y + y) * p.X + x;
-    const float rho = p.in0[node], T = p.in2[node];
-    const float ux = p.in1[node];
-    const float uy = (D >= 2) ? p.in1[p.N + node] : 0.f;
-    const float uz = (D >= 3) ? p.in1[2 * p.N + node] : 0.f;
-    const EqCoef k = eq_coef<D>(T, ux * ux + uy * uy + uz * uz, rho);
-    // the record of node `at` (per-node reference storage), from its own fields
-    auto record = [&](int64_t at) {
-        const float r0 = p.in0[at];
-        return make_float4(r0 - 1.0f, 0.5f * (r0 * (p.in2[at] - 1.0f)), r0 * (p.r * p.in1[at]),
-                           (D >= 2) ? r0 * (p.r * p.in1[p.N + at]) : 0.f);
-    };
-    // population i at the destination (dx, dy, dz)
-    auto put = [&](int i, int dx, int dy, int dz, float v) {
-        const int off = (dz * p.Y + dy) * p.pitch + dx;
-        if constexpr (is_node) st_ref(p, i, off, v, record(((int64_t)dz * p.Y + dy) * p.X + dx));
-        else st(p, i, off, v);
-    };
+    const InitSource n = init_source<LAT>(p, x, y, z);
+    const EqCoef &k = n.k;
+    const float ux = n.ux, uy = n.uy, uz = n.uz, T = n.T;
+    auto put = [&](int i, int dx, int dy, int dz, float v) { init_put<LAT>(p, i, dx, dy, dz, v); };
     // (the same branch for the whole launch: a copy axis anywhere)
     const bool open = MODE == 0 && (p.bc0 != 0 || (D >= 2 && p.bc1 != 0) || (D >= 3 && p.bc2 != 0));
     // the one destination of each population (-1: outside a copy axis)
@@ -957,49 +1006,19 @@ __device__ __forceinline__ void init_node(const Params<Lattice<LAT>::Q, ST> &p, 
         body(std::false_type{});
     } else {
         body(std::true_type{});
-        // the further destinations of a node on a copy axis's end, for the
-        // velocities that point out of it
-        const bool xl = p.bc0 != 0 && x == 0, xh = p.bc0 != 0 && x == p.X - 1;
-        const bool yl = D >= 2 && p.bc1 != 0 && y == 0, yh = D >= 2 && p.bc1 != 0 && y == p.Y - 1;
-        const bool zl = D >= 3 && p.bc2 != 0 && z == 0, zh = D >= 3 && p.bc2 != 0 && z == p.Z - 1;
-        auto spread = [&](int i, int ex, int ey, int ez) {
-            if (!((xl && ex < 0) || (xh && ex > 0) || (yl && ey < 0) || (yh && ey > 0) || (zl && ez < 0) ||
-                  (zh && ez > 0)))
-                return;
-            const PreImage rx = preimage(x, ex, p.X, p.bc0);
-            const PreImage ry = (D >= 2) ? preimage(y, ey, p.Y, p.bc1) : PreImage{0, 0};
-            const PreImage rz = (D >= 3) ? preimage(z, ez, p.Z, p.bc2) : PreImage{0, 0};
-            const float c = p.r * ((float)ex * ux + (float)ey * uy + (float)ez * uz);
-            const float v = p.w[i] * eq_single(k, c, p.r2 * (float)(ex * ex + ey * ey + ez * ez));
-#pragma unroll 1
-            for (int dz = rz.lo; dz <= rz.hi; ++dz)
-#pragma unroll 1
-                for (int dy = ry.lo; dy <= ry.hi; ++dy)
-#pragma unroll 1
-                    for (int dx = rx.lo; dx <= rx.hi; ++dx) put(i, dx, dy, dz, v);
-        };
-        if (xl || xh || yl || yh || zl || zh) {
-            // (7 populations unrolled: the ensemble's parameters are a
-            // register copy, which a run-time index would send to local
-            // memory; 37 and 49 unrolled cost more in cold instructions than
-            // the loops do, and so does a velocity table in cold memory)
-            if constexpr (Q == 7) {
-                static_for<0, Q>([&](auto ic) { spread(decltype(ic)::value, L::ex(decltype(ic)::value), 0, 0); });
-            } else {
-                int i = 0;
-#pragma unroll 1
-                for (int ez = (D >= 3) ? -3 : 0; ez <= ((D >= 3) ? 3 : 0); ++ez)
-#pragma unroll 1
-                    for (int ey = -3; ey <= 3; ++ey)
-#pragma unroll 1
-                        for (int ex = -3; ex <= 3; ++ex)
-                            if (Q != 37 || d2q37_member(ex, ey)) spread(i++, ex, ey, ez);
-            }
+        // (the other lattices' further destinations: init_end_row.  Unrolled: the
+        // ensemble's parameters are a register copy, which a run-time index
+        // would send to local memory)
+        if constexpr (Q == 7) {
+            if (x == 0 || x == p.X - 1)
+                static_for<0, Q>([&](auto ic) {
+                    init_spread<LAT>(p, n, x, y, z, decltype(ic)::value, L::ex(decltype(ic)::value), 0, 0);
+                });
         }
     }
     float4 rc = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (is_node) {  // the node's reference: its own initial fields
-        rc = record(node);
+        rc = init_record<LAT>(p, n.node);
         p.ref_dst[self] = rc;
     }
     if (ROT) {
@@ -1013,12 +1032,84 @@ __device__ __forceinline__ void init_node(const Params<Lattice<LAT>::Q, ST> &p, 
     }
 }
 
+// The further destinations of the populations (., ey, ez) of a node on an end of
+// a copy axis.
+template <int LAT, typename ST>
+__device__ __forceinline__ void init_end_row(const Params<Lattice<LAT>::Q, ST> &p, int x, int y, int z, int ey, int ez)
+{
+    constexpr int Q = Lattice<LAT>::Q;
+    const InitSource n = init_source<LAT>(p, x, y, z);
+    int i = 0;
+    if constexpr (Q == 37) {
+        for (int q = 0; q < 7 * (ey + 3); ++q) i += d2q37_member(q % 7 - 3, q / 7 - 3);
+    } else {
+        i = ((Q == 343 ? (ez + 3) * 7 : 0) + ey + 3) * 7;
+    }
+#pragma unroll 1
+    for (int ex = -3; ex <= 3; ++ex)
+        if (Q != 37 || d2q37_member(ex, ey)) init_spread<LAT>(p, n, x, y, z, i++, ex, ey, ez);
+}
+
+// In two dimensions the grid's z counts 1 + 7: plane 0 is the nodes, the others
+// the rows e_y of the nodes on an end (one thread doing all the rows is a chain
+// of 49 populations that the rest of a small grid waits for).
 template <int LAT, bool ROT, int MODE, typename ST>
 __global__ void __launch_bounds__(kBlockX) k_init(const Params<Lattice<LAT>::Q, ST> p)
 {
     const int x = blockIdx.x * kBlockX + threadIdx.x;
     if (x >= p.X) return;
-    init_node<LAT, ROT, MODE>(p, x, blockIdx.y, blockIdx.z);
+    if constexpr (Lattice<LAT>::D == 2) {
+        const int y = blockIdx.y, row = blockIdx.z;
+        if (row > 0) {
+            if ((p.bc0 != 0 && (x == 0 || x == p.X - 1)) || (p.bc1 != 0 && (y == 0 || y == p.Y - 1)))
+                init_end_row<LAT>(p, x, y, 0, row - 4, 0);
+            return;
+        }
+        init_node<LAT, ROT, MODE>(p, x, y, 0);
+    } else {
+        init_node<LAT, ROT, MODE>(p, x, blockIdx.y, blockIdx.z);
+    }
+}
+
+// Nodes on an end of a copy axis in three dimensions, counted through: the ends
+// in z, then those in y of the other planes, then those in x of the other rows.
+struct Ends {
+    int ends[3], inner0[3], inner[3];  // nodes on the axis's ends; first and number of the others
+    int64_t z, y, x;                   // nodes of the three groups
+};
+inline Ends box_ends(const int n[3], const int bc[3])
+{
+    Ends e;
+    for (int a = 0; a < 3; ++a) {
+        e.ends[a] = bc[a] == 0 ? 0 : n[a] == 1 ? 1 : 2;
+        e.inner0[a] = bc[a] != 0;
+        e.inner[a] = n[a] - e.ends[a];
+    }
+    e.z = (int64_t)e.ends[2] * n[1] * n[0];
+    e.y = (int64_t)e.inner[2] * e.ends[1] * n[0];
+    e.x = (int64_t)e.inner[2] * e.inner[1] * e.ends[0];
+    return e;
+}
+// One thread per such node and row (., e_y, e_z) = blockIdx.y of populations.
+// (All 343 in the node's own thread, whose warp waits for it: initial state of
+// 24^3 float, open in x, 306 us, now 31, and 28 of the periodic box; 100 x 100 x 96
+// half, open in x and y, 2.2 ms, now 0.60.)
+template <int LAT, typename ST>
+__global__ void __launch_bounds__(kBlockX) k_init_ends(const Params<Lattice<LAT>::Q, ST> p, const Ends e)
+{
+    int64_t q = blockIdx.x * (int64_t)kBlockX + threadIdx.x;
+    int x, y, z;
+    if (q < e.z) {
+        x = (int)(q % p.X), y = (int)(q / p.X % p.Y), z = q / p.X / p.Y ? p.Z - 1 : 0;
+    } else if ((q -= e.z) < e.y) {
+        x = (int)(q % p.X), z = e.inner0[2] + (int)(q / p.X % e.inner[2]), y = q / p.X / e.inner[2] ? p.Y - 1 : 0;
+    } else if ((q -= e.y) < e.x) {
+        y = e.inner0[1] + (int)(q % e.inner[1]), z = e.inner0[2] + (int)(q / e.inner[1] % e.inner[2]);
+        x = q / e.inner[1] / e.inner[2] ? p.X - 1 : 0;
+    } else {
+        return;
+    }
+    init_end_row<LAT>(p, x, y, z, (int)blockIdx.y % 7 - 3, (int)blockIdx.y / 7 - 3);
 }
 
 // ---------------------------------------------------------------------------
@@ -1254,7 +1345,18 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
             return launch_pdl(k_step<LAT, ROT, MODE, ST>, grid, block, 0, s, p);
         }
         break;
-    case Op::Init: k_init<LAT, ROT, MODE><<<grid, block, 0, s>>>(p); break;
+    case Op::Init: {
+        const bool open = MODE == 0 && Lattice<LAT>::D >= 2 && (a.bc[0] || a.bc[1] || (Lattice<LAT>::D == 3 && a.bc[2]));
+        k_init<LAT, ROT, MODE><<<Lattice<LAT>::D == 2 && open ? dim3(grid.x, grid.y, 8) : grid, block, 0, s>>>(p);
+        if constexpr (Lattice<LAT>::D == 3 && MODE == 0) {
+            if (open) {
+                const int n[3] = {a.X, a.Y, a.Z};
+                const Ends e = box_ends(n, a.bc);
+                k_init_ends<LAT><<<dim3((unsigned)((e.z + e.y + e.x + kBlockX - 1) / kBlockX), 49), block, 0, s>>>(p, e);
+            }
+        }
+        break;
+    }
     case Op::Moments:
         if constexpr (pair_form<LAT, MODE, ST>()) {
             if (pair_whole(a)) k_moments_pair<LAT, ROT, true><<<pairs, block, 0, s>>>(p);
