@@ -264,30 +264,30 @@ __device__ __forceinline__ void q343_collide(const Params<kQ343> &p, const Q343W
 // shared memory for pass 2, which reaches them last, when L1 has long evicted
 // them; it works on the same stored bits, so the depth does not change
 // results.  Bound by load latency and issue at the resident warps (255
-// registers).  256^3 half, n = 0 / n = 4, ms per step, by threads per block,
-// stash planes and resident blocks per SM: 64, 4, 4: 7.69 / 8.60 (kept); 64,
-// 5, 3: 8.11 / 9.48; 64, 6, 3: 9.35 / 9.96; 64, 3, 6: 8.82 / 9.46; 128, 3, 3:
-// 7.75 / 8.55; 128, 0, 3: 8.41 / 9.71; one node per thread (128, 6, 3):
-// 8.22 / 9.48.
-#ifndef LBM_Q343_PAIR_BLOCK
-#define LBM_Q343_PAIR_BLOCK 64
-#endif
+// registers: eight warps an SM).  256^3 half, n = 0 / n = 4, ms per step, by
+// threads per block, stash planes and resident blocks per SM: 64, 4, 4: 7.69 /
+// 8.60 (kept); 64, 5, 3: 8.11 / 9.48; 64, 6, 3: 9.35 / 9.96; 64, 3, 6: 8.82 /
+// 9.46; 128, 3, 3: 7.75 / 8.55; 128, 0, 3: 8.41 / 9.71; 32, 4, 8: 8.33 / 9.36; one
+// node per thread (128, 6, 3): 8.22 / 9.48.
+//
+// A block is part of a row, so rows of an odd number of warps (2 x 32 nodes each)
+// take blocks of one warp: in blocks of two the last warp has no nodes and keeps
+// its registers.  us per step, n = 4, in blocks of 32 / 64: 36 x 36 x 25 33 / 54 (47
+// with one node per thread), 64 x 60 x 58 119 / 207 (190), 131 x 128 x 120 1718 /
+// 2068 (2547); even rows 78 x 82 x 72 415 / 371, 128^3 1118 / 975.
 #ifndef LBM_Q343_PAIR_STASH
 #define LBM_Q343_PAIR_STASH 4
 #endif
-#ifndef LBM_Q343_PAIR_MIN_BLOCKS
-#define LBM_Q343_PAIR_MIN_BLOCKS 4
-#endif
-constexpr int kPairBlock = LBM_Q343_PAIR_BLOCK;
+constexpr int kPairWarps = 8;  // resident warps per SM that the registers allow
 constexpr int kPairStash = LBM_Q343_PAIR_STASH;
-constexpr size_t kPairStashBytes = (size_t)kPairStash * 49 * kPairBlock * 4;
+template <int BLOCK> constexpr size_t pair_stash_bytes() { return (size_t)kPairStash * 49 * BLOCK * 4; }
 
 struct Q343PairSums {
     F2 rho, jx, jy, jz, e2;
 };
 
 // q343_sums of both nodes.
-template <int NS, bool WHOLE, typename ST>
+template <int NS, int BLOCK, bool WHOLE, typename ST>
 __device__ __forceinline__ Q343PairSums q343_pair_sums(const Params<kQ343, ST> &p, const PairOffsets &o, int z,
                                                        uint32_t *stash)
 {
@@ -307,7 +307,7 @@ __device__ __forceinline__ Q343PairSums q343_pair_sums(const Params<kQ343, ST> &
             for (int a = 0; a < 7; ++a) {
                 const int i = (c * 7 + b) * 7 + a;
                 const uint32_t v = ld_pair<WHOLE>(p, i, row, o, 3 - a);
-                if constexpr (KEEP) stash[i * kPairBlock + threadIdx.x] = v;
+                if constexpr (KEEP) stash[i * BLOCK + threadIdx.x] = v;
                 const F2 w = f2(p.w[i]);
                 const F2 g = fma2(w, Pair16<ST>::get(v), w);
                 cs[a] = add2(cs[a], g);
@@ -392,8 +392,8 @@ __device__ __forceinline__ void pair_quartic(const PairQuartic &q, float r2f, F2
     }
 }
 
-// q343_collide_dev of both nodes.
-template <bool ROT, int NS, bool WHOLE, typename ST>
+// q343_collide of both nodes, on deviations.
+template <bool ROT, int NS, int BLOCK, bool WHOLE, typename ST>
 __device__ __forceinline__ void q343_pair_collide(const Params<kQ343, ST> &p, const Q343Weights &qw,
                                                   const PairOffsets &o, int x, int z, const Q343PairSums &s,
                                                   const uint32_t *stash)
@@ -446,7 +446,7 @@ __device__ __forceinline__ void q343_pair_collide(const Params<kQ343, ST> &p, co
                     rx = fma2(f2(qw.w2x[b * 7 + a]), P, rx);
                 }
                 uint32_t d;
-                if constexpr (KEPT) d = stash[i * kPairBlock + threadIdx.x];
+                if constexpr (KEPT) d = stash[i * BLOCK + threadIdx.x];
                 else d = ld_pair<WHOLE>(p, i, row, o, 3 - a);
                 if (ex * ex + ey * ey <= 1 && ex * ex + ey * ey + ez * ez <= 1) {
                     if (ex == 0 && ey == 0 && ez == 0) { P_c = P; d_c = d; }
@@ -509,18 +509,18 @@ __device__ __forceinline__ void q343_pair_collide(const Params<kQ343, ST> &p, co
     }
 }
 
-template <bool ROT, bool WHOLE, typename ST>
-__global__ void __launch_bounds__(kPairBlock, LBM_Q343_PAIR_MIN_BLOCKS)
+template <bool ROT, int BLOCK, bool WHOLE, typename ST>
+__global__ void __launch_bounds__(BLOCK, kPairWarps * 32 / BLOCK)
     k_step_q343_pair(const Params<kQ343, ST> p, const Q343Weights qw)
 {
-    const int x = 2 * (blockIdx.x * kPairBlock + threadIdx.x);
+    const int x = 2 * (blockIdx.x * BLOCK + threadIdx.x);
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.X) return;
     const PairOffsets o = pair_offsets(p, x, y);
     extern __shared__ unsigned char q343_smem[];
     uint32_t *stash = reinterpret_cast<uint32_t *>(q343_smem);
-    const Q343PairSums s = q343_pair_sums<kPairStash, WHOLE>(p, o, z, stash);
-    q343_pair_collide<ROT, kPairStash, WHOLE>(p, qw, o, x, z, s, stash);
+    const Q343PairSums s = q343_pair_sums<kPairStash, BLOCK, WHOLE>(p, o, z, stash);
+    q343_pair_collide<ROT, kPairStash, BLOCK, WHOLE>(p, qw, o, x, z, s, stash);
 }
 
 template <bool ROT, bool WHOLE, typename ST>
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(kQ343Block, 4) k_moments_q343_pair(const Param
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.X) return;
     const PairOffsets o = pair_offsets(p, x, y);
-    const Q343PairSums s = q343_pair_sums<0, WHOLE>(p, o, z, nullptr);
+    const Q343PairSums s = q343_pair_sums<0, 0, WHOLE>(p, o, z, nullptr);
     F2 h[7];
     Moments m[2];
     q343_pair_moments<ROT, WHOLE>(p, o, z * p.pitch * p.Y + o.y[3], s, h, m[0], m[1]);
@@ -629,15 +629,21 @@ template <bool ROT, typename ST> cudaError_t launch_step_q343(const Args &a, cud
         k_step_q343<ROT><<<grid, kQ343Block, 0, s>>>(p, qw);
         return cudaGetLastError();
     } else {
-        const dim3 grid((a.X + 2 * kPairBlock - 1) / (2 * kPairBlock), a.Y, a.Z);
-        auto go = [&](auto whole) {
+        auto go = [&](auto whole, auto block) {
             constexpr bool W = decltype(whole)::value;
-            const cudaError_t e = allow_smem<k_step_q343_pair<ROT, W, ST>>(kPairStashBytes);
+            constexpr int B = decltype(block)::value;
+            constexpr size_t smem = pair_stash_bytes<B>();
+            const cudaError_t e = allow_smem<k_step_q343_pair<ROT, B, W, ST>>(smem);
             if (e != cudaSuccess) return e;
-            k_step_q343_pair<ROT, W, ST><<<grid, kPairBlock, kPairStashBytes, s>>>(p, qw);
+            const dim3 grid((a.X + 2 * B - 1) / (2 * B), a.Y, a.Z);
+            k_step_q343_pair<ROT, B, W, ST><<<grid, B, smem, s>>>(p, qw);
             return cudaGetLastError();
         };
-        return pair_whole(a) ? go(std::true_type{}) : go(std::false_type{});
+        const bool odd = (a.X + 63) / 64 % 2;
+        using B32 = std::integral_constant<int, 32>;
+        using B64 = std::integral_constant<int, 64>;
+        if (pair_whole(a)) return odd ? go(std::true_type{}, B32{}) : go(std::true_type{}, B64{});
+        return odd ? go(std::false_type{}, B32{}) : go(std::false_type{}, B64{});
     }
 }
 
