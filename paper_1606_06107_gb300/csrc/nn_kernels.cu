@@ -1556,9 +1556,10 @@ __global__ void __launch_bounds__(256) k_head_bwd(const float *gout, const __nv_
 // R = blockDim / C groups of C threads take the block's positions in turn
 // (thread = channel, the features broadcast from shared memory), their sums
 // meet in shared memory and leave as one coalesced reduction per block.
-// Bound by the read of gx0; with one strided reduction per thread and the
-// features read through L1 it was latency and same-address traffic: 27 us at
-// 2^15 positions, C = 128, F = 16 (82 before).
+// Bound by the read of gx0, eight loads of which a thread has in flight (a loop
+// left to the compiler's unrolling had one): 2^15 positions, C = 128, F = 16 16 us
+// (27, and 63 with one strided reduction per thread and the features read
+// through L1); 2^20, C = 256, F = 4 175 us (405, 283).
 template <int F>
 __global__ void __launch_bounds__(1024) k_lift_bwd(const float *gx0, const float *feat, float *gWl, float *gbl,
                                                    int64_t P, int C, int per_block)
@@ -1574,9 +1575,7 @@ __global__ void __launch_bounds__(1024) k_lift_bwd(const float *gx0, const float
     float acc[F], accb = 0.f;
 #pragma unroll
     for (int j = 0; j < F; ++j) acc[j] = 0.f;
-#pragma unroll 8
-    for (int q = r; q < n; q += R) {
-        const float g = gx0[(p0 + q) * C + c];
+    auto add = [&](int q, float g) {
         accb += g;
 #pragma unroll
         for (int j = 0; j < F / 4; ++j) {
@@ -1586,7 +1585,17 @@ __global__ void __launch_bounds__(1024) k_lift_bwd(const float *gx0, const float
             acc[4 * j + 2] = fmaf(g, f.z, acc[4 * j + 2]);
             acc[4 * j + 3] = fmaf(g, f.w, acc[4 * j + 3]);
         }
+    };
+    const float *g0 = gx0 + p0 * C + c;
+    int q = r;
+    for (; q + 7 * R < n; q += 8 * R) {  // eight loads in flight
+        float g[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) g[k] = g0[(int64_t)(q + k * R) * C];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) add(q + k * R, g[k]);
     }
+    for (; q < n; q += R) add(q, g0[(int64_t)q * C]);
     __syncthreads();  // the features have been read
     for (int k = 0; k < R; ++k) {
         if (r == k) {
@@ -2274,13 +2283,14 @@ int lbm_nn_lift_backward(const float *gx0, const float *feat, float *gWl, float 
     if (!gx0 || !feat || !gWl || !gbl || P < 1 || C < 32 || C > 1024 || C % 32 ||
         (F != 4 && F != 8 && F != 16 && F != 32))
         return LBM_EINVAL;
-    // 128 positions a block keep two blocks on every SM from 2^15 positions
-    // on; more of them for larger P, so that the reductions stay few
-    const int64_t want = std::max<int64_t>(128, (P + 8 * 152 - 1) / (8 * 152));
+    // 32 positions a thread; more of them for larger P, so that the reductions
+    // stay few
+    const int groups = std::max(1, 512 / C);
+    const int64_t want = std::max<int64_t>(32 * groups, (P + 8 * 152 - 1) / (8 * 152));
     const int per_block = (int)std::min<int64_t>(want, 16384 / (F * 4) * 2);  // features: at most 32 KB
     const int64_t nblocks = (P + per_block - 1) / per_block;
     if (nblocks > 0x7fffffff) return LBM_EINVAL;
-    const int blocks = (int)nblocks, threads = C * std::max(1, 512 / C);
+    const int blocks = (int)nblocks, threads = C * groups;
     const size_t sh = sizeof(float) * std::max((size_t)per_block * F, (size_t)C * (F + 1));
     cudaStream_t s = (cudaStream_t)stream;
     // [C][F + 1] sums of 1024 channels and 32 features exceed 48 KB
@@ -2363,8 +2373,11 @@ int lbm_nn_bias_grad(const void *gz, float *gb, int64_t P, int C, void *stream)
 {
     if (!gz || !gb || P < 1 || C < 1) return LBM_EINVAL;
     if (C % kTile == 0 && C / kTile <= 65535 && aligned16(gz)) {
-        // about two blocks an SM, at least four rows a thread
-        const int64_t rows = std::max<int64_t>(64, (P * (C / kTile) + 303) / 304);
+        // two blocks an SM, at least four rows a thread; eight from 2^26 values
+        // on, which no longer come from L2 (2^20 x 256: 158 -> 85 us; 2^15 x 256
+        // 4.6, 5.0 with eight)
+        const int64_t blocks = P * C >= (1 << 26) ? 8 * 152 : 2 * 152;
+        const int64_t rows = std::max<int64_t>(64, (P * (C / kTile) + blocks - 1) / blocks);
         const dim3 grid((unsigned)((P + rows - 1) / rows), C / kTile);
         return launched(launch_pdl(k_colsum8, grid, 256, 0, (cudaStream_t)stream, (const __nv_bfloat16 *)gz, gb, P, C, rows));
     }
