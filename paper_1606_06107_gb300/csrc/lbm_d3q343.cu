@@ -502,7 +502,7 @@ __device__ __forceinline__ void q343_pair_collide(const Params<kQ343, ST> &p, co
 #pragma unroll
         for (int k = 0; k < 5; ++k) rz[k] = bc_wrap(z + k - 2, p.Z, p.bc2) * plane + o.y[3];
         auto load = [&](int j, int row) { return ld_pair<WHOLE>(p, kQ343 + j, row, o, 0); };
-        pair_rot_update<WHOLE, 3, ST>(
+        pair_rot_update<ST>(
             p, m0, m1, h, [&](int j, int d) { return ld_pair<WHOLE>(p, kQ343 + j, rest, o, d); },
             [&](int j, int a, int d) { return load(j, a == 1 ? z * plane + o.y[3 + d] : rz[2 + d]); },
             [&](int j, F2 f) { put(kQ343 + j, fma2(f, f2(p.iwr[j]), f2(-1.0f))); });

@@ -128,7 +128,7 @@ __device__ __forceinline__ uint32_t ld_pair(const Params<Q, ST> &p, int pop, int
     return __byte_perm(a, b, 0x5410);
 }
 
-// Pull of both nodes: the raw pairs (kept when G is given) and the moments.
+// Pull of both nodes: the raw pairs.
 template <int LAT, bool ROT, bool WHOLE, typename ST>
 __device__ __forceinline__ void pair_pull(const Params<Lattice<LAT>::Q, ST> &p, const PairOffsets &o, uint32_t *graw,
                                           uint32_t *hraw)
@@ -182,12 +182,12 @@ __device__ __forceinline__ void pair_moments(const Params<Lattice<LAT>::Q, ST> &
     m1 = make_moments<2, ROT>(p, hi(rho), hi(jx), hi(jy), 0.f, hi(e2), hi(R2));
 }
 
-// rot_advect and rot_store of both nodes.  along(j, d): the raw pair of h_j at
+// rot_advect and rot_store of both nodes in three dimensions.  along(j, d): the raw pair of h_j at
 // columns x + d, x + d + 1 of the nodes' own row; across(j, axis, d): the pair
 // of the row (axis 1) or plane (axis 2) d nodes further; put(j, f) stores.
 // The columns x - 2 .. x + 3 and four rows serve both signs of both nodes'
 // velocities, so nothing is loaded twice and no lane waits for another's sign.
-template <bool WHOLE, int D, typename ST, int Q, typename Along, typename Across, typename Put>
+template <typename ST, int Q, typename Along, typename Across, typename Put>
 __device__ __forceinline__ void pair_rot_update(const Params<Q, ST> &p, const Moments &m0, const Moments &m1,
                                                 const F2 *h, Along &&along, Across &&across, Put &&put)
 {
@@ -217,7 +217,7 @@ __device__ __forceinline__ void pair_rot_update(const Params<Q, ST> &p, const Mo
                          f2(p0 ? hi(h[j]) : hi(l), p1 ? lo(r) : lo(h[j])), adv);
         }
 #pragma unroll
-        for (int a = 1; a < D; ++a) {
+        for (int a = 1; a < 3; ++a) {
             const bool p0 = n0[a] >= 0.f, p1 = n1[a] >= 0.f;
             const F2 b2 = decode(across(j, a, -2)), b1 = decode(across(j, a, -1));
             const F2 t1 = decode(across(j, a, 1)), t2 = decode(across(j, a, 2));

@@ -36,6 +36,7 @@
 #include <cmath>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include "../../include/lbm.h"
 
@@ -2144,11 +2145,8 @@ int conv_common(int epi, const void *in, const void *w, const ConvArgs &a, int i
         if (sms < 1 || total >= (1ll << 31)) return LBM_ECUDA;
         const int grid = (int)std::min<int64_t>(total, sms);
         const int smem = tcn_smem_bytes(rows);
-        if (epi == kEpiForward)
-            return launched(launch_pdl(k_conv_tcn<kEpiForward>, dim3(grid), kPThreads, smem, s, ma, mw, a, tiles_l, tiles_m, (int)total, rows));
-        else
-            return launched(launch_pdl(k_conv_tcn<kEpiInputGrad>, dim3(grid), kPThreads, smem, s, ma, mw, a, tiles_l, tiles_m, (int)total, rows));
-        return launched(cudaGetLastError());
+        return launched(launch_pdl(epi == kEpiForward ? k_conv_tcn<kEpiForward> : k_conv_tcn<kEpiInputGrad>,
+                                   dim3(grid), kPThreads, smem, s, ma, mw, a, tiles_l, tiles_m, (int)total, rows));
     }
     if (!map_act(&ma, in, a.B, a.L, a.C, kTile) || !map_w(&mw, w, a.C, a.k)) return LBM_ECUDA;
     const int tiles_l = (a.L + kTile - 1) / kTile, tiles_n = a.C / kTile;
@@ -2164,11 +2162,8 @@ int conv_common(int epi, const void *in, const void *w, const ConvArgs &a, int i
     const int sms = sm_count();
     if (sms < 1 || total >= (1ll << 31)) return LBM_ECUDA;
     const int grid = (int)std::min<int64_t>(total, sms);
-    if (epi == kEpiForward)
-        return launched(launch_pdl(k_conv_tcp<kEpiForward>, dim3(grid), kPThreads, kPSmemBytes, s, ma, mw, a, tiles_l, tiles_n, (int)total));
-    else
-        return launched(launch_pdl(k_conv_tcp<kEpiInputGrad>, dim3(grid), kPThreads, kPSmemBytes, s, ma, mw, a, tiles_l, tiles_n, (int)total));
-    return launched(cudaGetLastError());
+    return launched(launch_pdl(epi == kEpiForward ? k_conv_tcp<kEpiForward> : k_conv_tcp<kEpiInputGrad>, dim3(grid),
+                               kPThreads, kPSmemBytes, s, ma, mw, a, tiles_l, tiles_n, (int)total));
 }
 
 }  // namespace
@@ -2274,7 +2269,6 @@ int lbm_nn_lift(const float *feat, const float *Wl, const float *bl, void *x0, i
     case 16: return launched(launch_pdl(k_lift<16>, dim3(blocks), C, sh, s, feat, Wl, bl, out, P, C, per_block));
     default: return launched(launch_pdl(k_lift<32>, dim3(blocks), C, sh, s, feat, Wl, bl, out, P, C, per_block));
     }
-    return launched(cudaGetLastError());
 }
 
 int lbm_nn_lift_backward(const float *gx0, const float *feat, float *gWl, float *gbl, int64_t P,
@@ -2304,7 +2298,6 @@ int lbm_nn_lift_backward(const float *gx0, const float *feat, float *gWl, float 
     case 16: return launched(launch_pdl(k_lift_bwd<16>, dim3(blocks), threads, sh, s, gx0, feat, gWl, gbl, P, C, per_block));
     default: return launched(launch_pdl(k_lift_bwd<32>, dim3(blocks), threads, sh, s, gx0, feat, gWl, gbl, P, C, per_block));
     }
-    return launched(cudaGetLastError());
 }
 
 int lbm_nn_head(const void *x, const float *Wp, const float *bp, float *out, int64_t P, int C, int Fo,
@@ -2325,16 +2318,13 @@ int lbm_nn_head(const void *x, const float *Wp, const float *bp, float *out, int
     const size_t sh = wbytes + (two ? 2 : 1) * row2;
     int rc = set_head_attrs();
     if (rc != LBM_OK) return rc;
-#define LBM_HEAD(FO)                                                                     \
-    do {                                                                                 \
-        return launched(launch_pdl(two ? k_head<FO, 2> : k_head<FO, 1>, dim3((int)nblocks), 128, sh, s, xb, Wp, bp, out, P, C)); \
-    } while (0)
-    if (Fo == 3) LBM_HEAD(3);
-    else if (Fo == 6) LBM_HEAD(6);
-    else if (Fo == 12) LBM_HEAD(12);
-    else LBM_HEAD(24);
-#undef LBM_HEAD
-    return launched(cudaGetLastError());
+    auto go = [&](auto kernel) {
+        return launched(launch_pdl(kernel, dim3((int)nblocks), 128, sh, s, xb, Wp, bp, out, P, C));
+    };
+    if (Fo == 3) return two ? go(k_head<3, 2>) : go(k_head<3, 1>);
+    if (Fo == 6) return two ? go(k_head<6, 2>) : go(k_head<6, 1>);
+    if (Fo == 12) return two ? go(k_head<12, 2>) : go(k_head<12, 1>);
+    return two ? go(k_head<24, 2>) : go(k_head<24, 1>);
 }
 
 int lbm_nn_head_backward(const float *gout, const void *x, const float *Wp, const void *z, float *gx,
@@ -2350,23 +2340,17 @@ int lbm_nn_head_backward(const float *gout, const void *x, const float *Wp, cons
     auto xb = (const __nv_bfloat16 *)x;
     auto zb = (const __nv_bfloat16 *)z;
     auto gzb = (__nv_bfloat16 *)gz;
-#define LBM_HEAD_BWD(NJ, FO)                                                                          \
-    do {                                                                                              \
-        return launched(launch_pdl(vec ? k_head_bwd<NJ, FO, true> : k_head_bwd<NJ, FO, false>, dim3(grid), 256, 0, s, gout, xb, Wp, zb, gx, gzb, gWp, gbp, P)); \
-    } while (0)
-    if (C == 128) {
-        if (Fo == 3) LBM_HEAD_BWD(4, 3);
-        else if (Fo == 6) LBM_HEAD_BWD(4, 6);
-        else if (Fo == 12) LBM_HEAD_BWD(4, 12);
-        else LBM_HEAD_BWD(4, 24);
-    } else {
-        if (Fo == 3) LBM_HEAD_BWD(8, 3);
-        else if (Fo == 6) LBM_HEAD_BWD(8, 6);
-        else if (Fo == 12) LBM_HEAD_BWD(8, 12);
-        else LBM_HEAD_BWD(8, 24);
-    }
-#undef LBM_HEAD_BWD
-    return launched(cudaGetLastError());
+    auto go = [&](auto kernel) {
+        return launched(launch_pdl(kernel, dim3(grid), 256, 0, s, gout, xb, Wp, zb, gx, gzb, gWp, gbp, P));
+    };
+    auto with = [&](auto nj) {
+        constexpr int NJ = decltype(nj)::value;
+        if (Fo == 3) return vec ? go(k_head_bwd<NJ, 3, true>) : go(k_head_bwd<NJ, 3, false>);
+        if (Fo == 6) return vec ? go(k_head_bwd<NJ, 6, true>) : go(k_head_bwd<NJ, 6, false>);
+        if (Fo == 12) return vec ? go(k_head_bwd<NJ, 12, true>) : go(k_head_bwd<NJ, 12, false>);
+        return vec ? go(k_head_bwd<NJ, 24, true>) : go(k_head_bwd<NJ, 24, false>);
+    };
+    return C == 128 ? with(std::integral_constant<int, 4>{}) : with(std::integral_constant<int, 8>{});
 }
 
 int lbm_nn_bias_grad(const void *gz, float *gb, int64_t P, int C, void *stream)
@@ -2445,9 +2429,7 @@ int lbm_nn_features(const float *rho, const float *u, const float *T, const floa
     cudaStream_t s = (cudaStream_t)stream;
     if (n >= kVecNodes && L % 4 == 0 && aligned16(rho) && aligned16(u) && aligned16(T))
         return launched(launch_pdl(k_features<true>, dim3(grid_for(n / 4)), 256, 0, s, rho, u, T, gamma, feat, n, L, sc));
-    else
-        return launched(launch_pdl(k_features<false>, dim3(grid_for(n)), 256, 0, s, rho, u, T, gamma, feat, n, L, sc));
-    return launched(cudaGetLastError());
+    return launched(launch_pdl(k_features<false>, dim3(grid_for(n)), 256, 0, s, rho, u, T, gamma, feat, n, L, sc));
 }
 
 int lbm_nn_targets(const float *rho, const float *u, const float *T, const float *rho2,
@@ -2461,9 +2443,7 @@ int lbm_nn_targets(const float *rho, const float *u, const float *T, const float
     if (n >= kVecNodes && n % 4 == 0 && aligned16(rho) && aligned16(u) && aligned16(T) && aligned16(rho2) && aligned16(u2) &&
         aligned16(T2) && aligned16(target))
         return launched(launch_pdl(k_targets<true>, dim3(grid_for(n / 4)), 256, 0, s, rho, u, T, rho2, u2, T2, target, n, sc));
-    else
-        return launched(launch_pdl(k_targets<false>, dim3(grid_for(n)), 256, 0, s, rho, u, T, rho2, u2, T2, target, n, sc));
-    return launched(cudaGetLastError());
+    return launched(launch_pdl(k_targets<false>, dim3(grid_for(n)), 256, 0, s, rho, u, T, rho2, u2, T2, target, n, sc));
 }
 
 int lbm_nn_apply(const float *rho, const float *u, const float *T, const float *out, float *rho2,
@@ -2476,9 +2456,7 @@ int lbm_nn_apply(const float *rho, const float *u, const float *T, const float *
     if (n >= kVecNodes && n % 4 == 0 && aligned16(rho) && aligned16(u) && aligned16(T) && aligned16(rho2) && aligned16(u2) &&
         aligned16(T2) && aligned16(out))
         return launched(launch_pdl(k_apply<true>, dim3(grid_for(n / 4)), 256, 0, s, rho, u, T, out, rho2, u2, T2, n, sc));
-    else
-        return launched(launch_pdl(k_apply<false>, dim3(grid_for(n)), 256, 0, s, rho, u, T, out, rho2, u2, T2, n, sc));
-    return launched(cudaGetLastError());
+    return launched(launch_pdl(k_apply<false>, dim3(grid_for(n)), 256, 0, s, rho, u, T, out, rho2, u2, T2, n, sc));
 }
 
 int lbm_nn_tube_checks(const float *rho, const float *u, const float *T, const float *rho2,
