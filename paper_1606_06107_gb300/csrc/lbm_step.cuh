@@ -52,12 +52,15 @@ template <typename ST, int MODE> struct StepMinBlocks {
     static constexpr int value = (std::is_same<ST, float>::value || MODE != 0) ? 4 : 5;
 #endif
 };
-// Float FD steps of more than one wave at four blocks per SM take the kernel
-// compiled for three (168 registers): they are bound by the latency of 4-7
-// loads per population from L2, and more of them in flight are worth more than
-// more warps.  600 x 420 D2Q37 38.1 -> 30.6 us, 2048 x 1024 D2Q49 367 -> 285; a
-// single wave loses (300 x 200 D2Q49, n = 0, 600 blocks: 10.3 -> 11.4), and five
-// or six blocks spill (50.5 / 53.7 us at 600 x 420).
+// Float FD steps are compiled for three blocks per SM too (168 registers): they
+// are bound by the latency of 4-7 loads per population from L2, and more of them
+// in flight are worth more than more warps.  All grids take that kernel but those
+// of one wave at four blocks per SM and two at three, where it loses, unless its
+// registers also save spills (D2Q49 with rotation).  us per step, four / three
+// blocks: 40 x 16 D2Q37 n = 3 7.4 / 5.0, D2Q49 n = 3 14.9 / 6.9; 600 blocks D2Q37
+// n = 0 8.1 / 9.5, n = 3 10.0 / 11.0, D2Q49 n = 0 11.3 / 12.2, n = 3 18.9 / 14.7; 600
+// x 420 D2Q37 n = 3 38.1 / 31.0.  Two blocks 34.1 / 312 at 600 x 420 and 2048 x 1024
+// (30.6 / 285); five or six spill (50.5 / 53.7 at 600 x 420).
 #ifndef LBM_FD_WIDE_BLOCKS
 #define LBM_FD_WIDE_BLOCKS 3
 #endif
@@ -1338,11 +1341,14 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
             // per-node references: the deviation-space kernel (STREAM only)
             return launch_pdl(k_step_node<LAT, ROT, ST>, grid, block, 0, s, p);
         } else {
-            if constexpr (MODE == 1 && std::is_same<ST, float>::value && Lattice<LAT>::D == 2) {
-                if ((int64_t)grid.x * grid.y > 4 * (int64_t)device_sms())
+            constexpr bool wide = MODE == 1 && std::is_same<ST, float>::value && Lattice<LAT>::D == 2;
+            if constexpr (wide) {
+                const int64_t blocks = (int64_t)grid.x * grid.y, sms = device_sms();
+                if ((LAT == 3 && ROT) || blocks <= 3 * sms || blocks > 4 * sms)
                     return launch_pdl(k_step<LAT, ROT, MODE, ST, kFdWideBlocks>, grid, block, 0, s, p);
             }
-            return launch_pdl(k_step<LAT, ROT, MODE, ST>, grid, block, 0, s, p);
+            if constexpr (!(wide && LAT == 3 && ROT))
+                return launch_pdl(k_step<LAT, ROT, MODE, ST>, grid, block, 0, s, p);
         }
         break;
     case Op::Init: {
