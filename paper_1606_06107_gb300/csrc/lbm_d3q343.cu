@@ -564,20 +564,67 @@ __global__ void __launch_bounds__(kQ343Block, LBM_Q343_MIN_BLOCKS)
     q343_collide<ROT>(p, qw, o, z, q343_sums(p, o, z));
 }
 
+// The five sums for the moments alone: by e_x, e_y and e_z first, opposite
+// velocities before the rest, as node_moments takes them (no sum has more than 49
+// terms in a row, and a mirror-symmetric state gives exactly zero momentum).
+__device__ __forceinline__ Q343Sums q343_moment_sums(const Params<kQ343> &p, const Offsets &o, int z)
+{
+    const int plane = p.pitch * p.Y;
+    float cs[7], rs[7];
+#pragma unroll
+    for (int a = 0; a < 7; ++a) cs[a] = rs[a] = 0.f;
+    auto add = [&](int c) {  // the sum of the plane of e_z = c - 3
+        const int zo = bc_wrap(z - (c - 3), p.Z, p.bc2) * plane;
+        float sum = 0.f;
+#pragma unroll
+        for (int b = 0; b < 7; ++b) {
+            const int row = zo + o.y[6 - b];
+            float rsum = 0.f;
+#pragma unroll
+            for (int a = 0; a < 7; ++a) {
+                const float g = q343_load(p, (c * 7 + b) * 7 + a, row + o.x[6 - a]);
+                cs[a] += g;
+                rsum += g;
+            }
+            rs[b] += rsum;
+            sum += rsum;
+        }
+        return sum;
+    };
+    Q343Sums s{0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int k = 3; k >= 1; --k) {
+        const float lo = add(3 - k), hi = add(3 + k), d = (float)k;
+        s.jz = fmaf(d, hi - lo, s.jz);
+        s.e2 = fmaf(d * d, hi + lo, s.e2);
+    }
+    add(3);
+    s.rho = cs[3];
+#pragma unroll
+    for (int k = 1; k <= 3; ++k) {
+        const float d = (float)k, sx = cs[3 + k] + cs[3 - k];
+        s.rho += sx;
+        s.jx = fmaf(d, cs[3 + k] - cs[3 - k], s.jx);
+        s.jy = fmaf(d, rs[3 + k] - rs[3 - k], s.jy);
+        s.e2 = fmaf(d * d, sx, s.e2);
+        s.e2 = fmaf(d * d, rs[3 + k] + rs[3 - k], s.e2);
+    }
+    return s;
+}
+
 // rho, u, T of the current state: pass 1 of the step and the rotational
 // energy, nothing kept (no stash, no per-node array of the 343 values: that
 // array, in local memory, is what the general k_moments spent its time on).
 // Bound by issue and load latency, as pass 1 of the step is: 101 x 96 x 90
 // float n = 4 0.241 ms (0.860 with k_moments); 256^3 half, two nodes per
-// thread below, 2.30 ms (3.12 with one, 14.6
-// with k_moments).
+// thread below, 2.30 ms (3.12 with one, 14.6 with k_moments).
 template <bool ROT> __global__ void __launch_bounds__(kQ343Block, 4) k_moments_q343(const Params<kQ343> p)
 {
     const int x = blockIdx.x * kQ343Block + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.X) return;
     const Offsets o = node_offsets<3>(p, x, y, z);
-    const Q343Sums s = q343_sums(p, o, z);
+    const Q343Sums s = q343_moment_sums(p, o, z);
     float R2 = 0.f;
     if (ROT) {
 #pragma unroll

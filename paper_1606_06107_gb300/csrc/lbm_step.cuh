@@ -835,9 +835,8 @@ __global__ void __launch_bounds__(kBlockX, MINB) k_step(const Params<Lattice<LAT
     auto store_all = [&] {
         static_for<0, Q>([&](auto ic) { st(p, decltype(ic)::value, o.self(), g[decltype(ic)::value]); });
     };
-    // With three blocks per SM the rotational loads too go before the stores
-    // (600 x 420: 33.2 -> 31.5 us); a single wave is better off with them after
-    // (100 x 60: 7.4 us, 8.3 before).
+    // With three blocks per SM the rotational loads too go before the stores (600
+    // x 420: 33.2 -> 31.5 us); with four there are no registers for it.
     constexpr bool STORE_LAST = FD && ROT && MINB == kFdWideBlocks;
     if constexpr (FD && !STORE_LAST) store_all();
     if (ROT) {

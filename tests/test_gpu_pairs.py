@@ -51,3 +51,16 @@ def test_moments_2d_are_those_of_the_state(kind, storage, shape, bc, n):
     got = [x.cpu().numpy().astype(np.float64).reshape(w.shape) for x, w in zip(sim.moments(), (rho, u, T))]
     for a, b, tol in zip(got, (rho, u, T), (3e-6, 4e-6, 1e-5)):
         assert np.abs(a - b).max() <= tol * rho.max(), np.abs(a - b).max()
+
+
+@pytest.mark.parametrize("n", [0, 4])
+def test_d3q343_float_moments_at_rest(n):
+    """Opposite velocities are combined before anything else: a uniform state at
+    rest has exactly no momentum."""
+    from paper_1606_06107_gb300 import Lbm
+    shape = (70, 4, 3)
+    N = int(np.prod(shape))
+    for rho, T in ((1.1, 0.9), (0.7, 1.3), (1.0, 1.01)):
+        sim = Lbm("D3Q343", n, 0.8, shape, ("periodic",) * 3)
+        sim.set_macro(np.full(N, rho), np.zeros((3, N)), np.full(N, T))
+        assert not sim.moments()[1].cpu().numpy().any()
