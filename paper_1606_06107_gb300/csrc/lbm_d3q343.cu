@@ -523,6 +523,56 @@ __global__ void __launch_bounds__(BLOCK, kPairWarps * 32 / BLOCK)
     q343_pair_collide<ROT, kPairStash, BLOCK, WHOLE>(p, qw, o, x, z, s, stash);
 }
 
+// The sums for the moments alone, opposite velocities before the rest
+// (q343_moment_sums below) of both nodes.
+template <bool WHOLE, typename ST>
+__device__ __forceinline__ Q343PairSums q343_pair_moment_sums(const Params<kQ343, ST> &p, const PairOffsets &o, int z)
+{
+    const int plane = p.pitch * p.Y;
+    F2 cs[7], rs[7];
+#pragma unroll
+    for (int a = 0; a < 7; ++a) cs[a] = rs[a] = f2(0.f);
+    auto add = [&](int c) {  // the sum of the plane of e_z = c - 3
+        const int zo = bc_wrap(z - (c - 3), p.Z, p.bc2) * plane;
+        F2 sum = f2(0.f);
+#pragma unroll
+        for (int b = 0; b < 7; ++b) {
+            const int row = zo + o.y[6 - b];
+            F2 rsum = f2(0.f);
+#pragma unroll
+            for (int a = 0; a < 7; ++a) {
+                const int i = (c * 7 + b) * 7 + a;
+                const F2 w = f2(p.w[i]);
+                const F2 g = fma2(w, Pair16<ST>::get(ld_pair<WHOLE>(p, i, row, o, 3 - a)), w);
+                cs[a] = add2(cs[a], g);
+                rsum = a ? add2(rsum, g) : g;
+            }
+            rs[b] = add2(rs[b], rsum);
+            sum = add2(sum, rsum);
+        }
+        return sum;
+    };
+    Q343PairSums s{f2(0.f), f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
+#pragma unroll 1
+    for (int k = 3; k >= 1; --k) {
+        const F2 lo = add(3 - k), hi = add(3 + k);
+        s.jz = fma2(f2((float)k), sub2(hi, lo), s.jz);
+        s.e2 = fma2(f2((float)(k * k)), add2(hi, lo), s.e2);
+    }
+    add(3);
+    s.rho = cs[3];
+#pragma unroll
+    for (int k = 1; k <= 3; ++k) {
+        const F2 d = f2((float)k), dd = f2((float)(k * k)), sx = add2(cs[3 + k], cs[3 - k]);
+        s.rho = add2(s.rho, sx);
+        s.jx = fma2(d, sub2(cs[3 + k], cs[3 - k]), s.jx);
+        s.jy = fma2(d, sub2(rs[3 + k], rs[3 - k]), s.jy);
+        s.e2 = fma2(dd, sx, s.e2);
+        s.e2 = fma2(dd, add2(rs[3 + k], rs[3 - k]), s.e2);
+    }
+    return s;
+}
+
 template <bool ROT, bool WHOLE, typename ST>
 __global__ void __launch_bounds__(kQ343Block, 4) k_moments_q343_pair(const Params<kQ343, ST> p)
 {
@@ -530,7 +580,7 @@ __global__ void __launch_bounds__(kQ343Block, 4) k_moments_q343_pair(const Param
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= p.X) return;
     const PairOffsets o = pair_offsets(p, x, y);
-    const Q343PairSums s = q343_pair_sums<0, 0, WHOLE>(p, o, z, nullptr);
+    const Q343PairSums s = q343_pair_moment_sums<WHOLE>(p, o, z);
     F2 h[7];
     Moments m[2];
     q343_pair_moments<ROT, WHOLE>(p, o, z * p.pitch * p.Y + o.y[3], s, h, m[0], m[1]);

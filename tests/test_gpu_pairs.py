@@ -54,13 +54,14 @@ def test_moments_2d_are_those_of_the_state(kind, storage, shape, bc, n):
 
 
 @pytest.mark.parametrize("n", [0, 4])
-def test_d3q343_float_moments_at_rest(n):
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+def test_d3q343_moments_at_rest(n, storage):
     """Opposite velocities are combined before anything else: a uniform state at
     rest has exactly no momentum."""
     from paper_1606_06107_gb300 import Lbm
     shape = (70, 4, 3)
     N = int(np.prod(shape))
     for rho, T in ((1.1, 0.9), (0.7, 1.3), (1.0, 1.01)):
-        sim = Lbm("D3Q343", n, 0.8, shape, ("periodic",) * 3)
+        sim = Lbm("D3Q343", n, 0.8, shape, ("periodic",) * 3, storage=storage)
         sim.set_macro(np.full(N, rho), np.zeros((3, N)), np.full(N, T))
         assert not sim.moments()[1].cpu().numpy().any()
