@@ -102,7 +102,8 @@ __device__ __forceinline__ Params<7> tube_params(const BatchParams &bp, const Tu
 // buffers per step this reads and writes L2 once in sixteen steps, for 8-12 %
 // more nodes.
 //
-// Bound by shared-memory reads and the barriers between steps.  One node a
+// Bound by issue (81 % of the slots at 1024 x 384 nodes), shared-memory reads (LSU
+// 63 %) and the barriers between steps.  One node a
 // thread against two in packed arithmetic (f32x2, half a window apart), 32 FD
 // steps: 1024 tubes of 4096 nodes 1.78 / 2.01 ms, of 640 285 / 335 us, of 384 179
 // / 172, of 100-150 83 / 102; 152 tubes of 384 41 / 54, one of 100-150 30 / 45: a

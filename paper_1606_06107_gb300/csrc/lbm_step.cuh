@@ -1292,8 +1292,8 @@ template <auto KERNEL> cudaError_t allow_smem(size_t bytes)
 // running (programmatic dependent launch): `kernel` calls pdl_wait() before
 // its first global access, so only its launch and its index arithmetic
 // overlap the predecessor: what a step of a small grid waits for.  1000 x 16
-// D2Q37 6.1 -> 3.5 us per step, 600 x 420 FD 38.1 -> 36.5, 1021 x 771 node
-// reference 107 -> 103; a 2048^2 float step 318 -> 316.
+// D2Q37 6.26 -> 3.25 us per step, 500 x 100 D2Q49 8.3 -> 5.6, 1021 x 771 node
+// reference 110 -> 107; a 2048^2 float step 322 -> 317.
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args)
 {
