@@ -281,7 +281,7 @@ Args make_args(const lbm_ctx *h)
 
 cudaError_t launch(lbm_ctx *h, Op op, const Args &a)
 {
-    ++h->launches;
+    h->launches += op == Op::Init && lbm::init_has_ends(a) ? 2 : 1;
     switch (h->lattice) {
     case LBM_D1Q7: return lbm::launch_d1q7(op, a, h->stream);
     case LBM_D2Q37: return lbm::launch_d2q37(op, a, h->stream);

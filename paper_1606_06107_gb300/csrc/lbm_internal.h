@@ -49,6 +49,10 @@ cudaError_t launch_d2q37(Op op, const Args &a, cudaStream_t s);
 cudaError_t launch_d2q49(Op op, const Args &a, cudaStream_t s);
 cudaError_t launch_d3q343(Op op, const Args &a, cudaStream_t s);
 
+// Whether the initial state takes a second launch (k_init_ends): STREAM mode in
+// three dimensions with an open axis.
+inline bool init_has_ends(const Args &a) { return a.D == 3 && a.mode == 0 && (a.bc[0] || a.bc[1] || a.bc[2]); }
+
 // Many steps of one D1Q7 tube in one launch: from a.src to a.dst, which may
 // be the same buffer (lbm_d1q7.cu).
 bool tube_steps_ok(const Args &a, int64_t steps);

@@ -1351,10 +1351,10 @@ cudaError_t launch_mode(Op op, const Args &a, cudaStream_t s)
         }
         break;
     case Op::Init: {
-        const bool open = MODE == 0 && Lattice<LAT>::D >= 2 && (a.bc[0] || a.bc[1] || (Lattice<LAT>::D == 3 && a.bc[2]));
-        k_init<LAT, ROT, MODE><<<Lattice<LAT>::D == 2 && open ? dim3(grid.x, grid.y, 8) : grid, block, 0, s>>>(p);
+        const bool rows = Lattice<LAT>::D == 2 && MODE == 0 && (a.bc[0] || a.bc[1]);
+        k_init<LAT, ROT, MODE><<<rows ? dim3(grid.x, grid.y, 8) : grid, block, 0, s>>>(p);
         if constexpr (Lattice<LAT>::D == 3 && MODE == 0) {
-            if (open) {
+            if (init_has_ends(a)) {
                 const int n[3] = {a.X, a.Y, a.Z};
                 const Ends e = box_ends(n, a.bc);
                 k_init_ends<LAT><<<dim3((unsigned)((e.z + e.y + e.x + kBlockX - 1) / kBlockX), 49), block, 0, s>>>(p, e);

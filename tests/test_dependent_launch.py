@@ -72,3 +72,17 @@ def test_queued_steps_equal_single_ones(kind, shape, storage, mode):
         torch.cuda.synchronize()
     for x, y in zip(sims[0].state(), sims[1].state()):
         assert torch.equal(x, y)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind,shape,bc,init", [("D2Q37", (20, 10), ("copy", "copy"), 1), ("D3Q343", (9, 8, 7), ("periodic",) * 3, 1),
+                                                ("D3Q343", (9, 8, 7), ("periodic", "periodic", "copy"), 2)])
+def test_launch_count(kind, shape, bc, init):
+    from paper_1606_06107_gb300 import Lbm
+    wl = workloads.smooth_random(shape, seed=2, kind=kind, n=3)
+    sim = Lbm(kind, 3, wl.tau, shape, bc)
+    at = sim.launches
+    sim.set_macro(wl.rho, wl.u, wl.T)
+    assert sim.launches - at == init
+    sim.step(3)
+    assert sim.launches - at == init + 3
